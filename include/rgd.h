@@ -208,7 +208,8 @@ int rgd_prefix_decode_attn_noalloc(const rgd_attn_shape* shape, const rgd_bf16* 
  *   kept_mask uint8 [rows, vocab] or NULL: 1 where i in K (sample rows only;
  *     rows that are greedy or inactive are not written).
  * is_probe may be NULL (no probe rows); row_active may be NULL (all active).
- * vocab must satisfy vocab * element size <= 8 * 200 KiB. */
+ * vocab must satisfy vocab * element size <= 2 MiB.  A wait that gives up sets
+ * RGD_DEV_WAIT_TIMEOUT in dev_status; outputs of rows then are missing. */
 int rgd_sample_head(int32_t rows, int32_t vocab, int32_t dtype, const void* logits,
                     const uint8_t* is_probe, const float* temperature, const float* min_p,
                     const uint64_t* seed, uint64_t step, const uint8_t* row_active,
@@ -302,7 +303,9 @@ int rgd_sample_head_gated(int32_t rows, int32_t vocab, int32_t dtype, const void
  * step's rows, then rgd_sample_head_gated over the step's logits (two kernels
  * on `stream`; the head's blocks are scheduled while the attention finishes).
  * The logits are the caller's: the model between the attention output and the
- * next-token logits (projections, MLP, LM head) is not part of this library.
+ * next-token logits (projections, MLP, LM head) is not part of this library;
+ * the head reads its inputs while the attention finishes (the attention writes
+ * none of them).
  * Arguments are those of the two calls, with rows = num_groups *
  * rows_per_group and one row_active shared by both (the attention reads it,
  * the gate updates it); out and lse receive the attention output.  The first

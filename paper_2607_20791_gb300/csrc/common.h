@@ -37,6 +37,16 @@ int check_gated_head(const char* fn, int32_t rows, int32_t vocab, int32_t dtype,
                      const float* temperature, const float* min_p, const uint64_t* seed, const int32_t* token_out,
                      const rgd_trie* trie, int32_t rows_per_group, int32_t max_len, const rgd_gate_state* state);
 
+// rgd_sample_head_gated with its arguments checked under the name `fn`.  early:
+// the previous kernel on the stream neither writes an input of the head nor was
+// itself started before every input was complete, so the head may read them
+// before that kernel ends (it still waits for it before it writes anything).
+int launch_gated_head(const char* fn, int32_t rows, int32_t vocab, int32_t dtype, const void* logits,
+                      const uint8_t* is_probe, const float* temperature, const float* min_p, const uint64_t* seed,
+                      uint64_t step, uint8_t* row_active, int32_t* token_out, int32_t* kept_count,
+                      const rgd_trie* trie, int32_t rows_per_group, int32_t eos_token, int32_t max_len,
+                      rgd_gate_state* state, int32_t* dev_status, rgd_stream_t stream, bool early);
+
 }  // namespace rgd
 
 #define RGD_CHECK_ARG(cond, ...)                                        \
