@@ -75,10 +75,10 @@ def algorithmic_bytes(case):
 
 # DRAM traffic of one attention launch on the Llama-3-8B-shaped step
 # (dram__bytes_read.sum + dram__bytes_write.sum), from one ncu capture of the
-# kernel sources whose hash is given (profiles/attn_t_kernel_llama8b.md has the
+# kernel sources whose hash is given (profiles/attn_kernel_llama8b.md has the
 # command); reported only while those sources are unchanged, else null.
 ATTN_TRAFFIC = {"sources_sha256": "adc56870d915", "bytes_per_launch": 121346048}
-ATTN_SOURCES = ("attention.cu", "attention_t.cuh")
+ATTN_SOURCES = ("attention.cu", "attention.h", "attention_kernel.cuh")
 
 
 def _kernel_hash():
@@ -855,7 +855,7 @@ def run_ours(args):
             "step_hbm_gbs": step_gbs, "step_hbm_frac": step_gbs / peak,
             "step_algorithmic_bytes": step_bytes,
             "kernels_ms": {"attention": mean_attn, "sample_head_with_gate": mean_hg},
-            "roofline": {"bound": "hbm", "kernel": "attn_t_kernel<128, 3>", "achieved": attn_gbs,
+            "roofline": {"bound": "hbm", "kernel": "attn_kernel<128, 3, 8>", "achieved": attn_gbs,
                          "peak": peak, "unit": "GB/s", "frac": attn_gbs / peak, "traffic": traffic,
                          "traffic_source": ("one ncu capture of these kernel sources (dram bytes read + written per "
                                             "launch), recorded in bench.py with the sources' hash"

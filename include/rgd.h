@@ -142,7 +142,9 @@ size_t rgd_prefix_decode_attn_workspace_size(const rgd_attn_shape* shape);
  *                      a call with J > 8192 moves the scratch, so zero-fill the
  *                      workspace whenever the shape changes across it.  Calls
  *                      that share a workspace must not overlap in time.
- * One kernel runs on `stream`.  A job split across blocks is merged by the
+ * One kernel runs on `stream`, launched as a programmatic dependent of the
+ * previous kernel on the stream (it is scheduled while that kernel finishes and
+ * waits for it before reading any input).  A job split across blocks is merged by the
  * block holding its first page, which waits (bounded) for the job's other
  * pieces; those are the first pieces of later blocks and wait on no other
  * block, so the wait ends as long as blocks start in index order (num_ctas

@@ -1,0 +1,12 @@
+// The attention kernel for head dimension 128 (one translation unit per head
+// dimension, compiled in parallel).
+#include "attention_kernel.cuh"
+
+namespace rgd {
+
+int launch_attn_d128(const CUtensorMap& tmK, const CUtensorMap& tmV, const AttnParams& p, int smem_bytes,
+                    cudaStream_t st) {
+  return launch_attn<128>(tmK, tmV, p, smem_bytes, st);
+}
+
+}  // namespace rgd

@@ -38,9 +38,9 @@ int check_gated_head(const char* fn, int32_t rows, int32_t vocab, int32_t dtype,
                      const rgd_trie* trie, int32_t rows_per_group, int32_t max_len, const rgd_gate_state* state);
 
 // rgd_sample_head_gated with its arguments checked under the name `fn`.  early:
-// the previous kernel on the stream neither writes an input of the head nor was
-// itself started before every input was complete, so the head may read them
-// before that kernel ends (it still waits for it before it writes anything).
+// the previous kernel on the stream writes no input of the head and lets it
+// start only once every input was complete, so the head may read them before
+// that kernel ends (it still waits for it before it writes anything).
 int launch_gated_head(const char* fn, int32_t rows, int32_t vocab, int32_t dtype, const void* logits,
                       const uint8_t* is_probe, const float* temperature, const float* min_p, const uint64_t* seed,
                       uint64_t step, uint8_t* row_active, int32_t* token_out, int32_t* kept_count,

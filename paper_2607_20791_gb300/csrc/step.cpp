@@ -23,8 +23,9 @@ extern "C" int rgd_decode_step(const rgd_attn_shape* shape, const rgd_bf16* q, c
                                       suffix_block_table, suffix_len, row_active, softmax_scale, out, lse,
                                       workspace, workspace_bytes, dev_status, stream))
     return rc;
-  // the head reads nothing that the attention writes, and the attention is an
-  // ordinary launch: its inputs were complete before the attention began
+  // the head reads nothing that the attention writes, and its blocks start only
+  // once every block of the attention has waited for the kernels before it: its
+  // inputs are complete by then
   return rgd::launch_gated_head("rgd_decode_step", (int32_t)rows, vocab, dtype, logits, is_probe, temperature, min_p,
                                 seed, step, row_active, token_out, kept_count, trie, shape->rows_per_group, eos_token,
                                 max_len, state, dev_status, stream, true);
