@@ -218,6 +218,8 @@ extern "C" int rgd_prefix_decode_attn(const rgd_attn_shape* shape, const rgd_bf1
   p.hv = pl.hv;
   p.np = pl.np;
   p.nqb = pl.nqb;
+  p.fold = std::min(kMaxFold, pl.hk * kGroupPages * kPage * s.head_dim * 2 /
+                                  (pl.nq * s.head_dim * 4 + ml_stride(pl.nq) * 8));
   p.slen_in_smem = pl.slen_in_smem ? 1 : 0;
   p.L = pl.layout;
   p.scale_log2 = softmax_scale * kLog2e;

@@ -15,6 +15,11 @@ namespace rgd {
 constexpr int kPage = 16;                      // tokens per KV page
 constexpr int kGroupPages = 8;                 // pages per group: 128 tokens, the MMA's M
 constexpr int kMaxQueries = 128;               // rows_per_group * Hq / Hkv
+// A split job of at most this many other pieces is folded in the merging block's K
+// ring.  With ten (a page each) the fold's loops took 17 us where the merge from
+// global memory by every thread takes 12; with one or two the fold saves 1.7 us of
+// 33 (16 groups x 5 rows) and 6 of 40 (200 x 16 rows, D 64).
+constexpr int kMaxFold = 4;
 constexpr int kRingMax = 4;                    // K or V areas at most
 constexpr int kSmemLimit = 226 * 1024;         // dynamic part; static shared memory needs the rest
 
@@ -52,7 +57,7 @@ __host__ __device__ constexpr int query_cols(int sets, int per_set) { return (se
 // Shared-memory carve-up, laid out by the host.  Rings, P^T and Q are
 // 1024-byte aligned (swizzle atoms).
 struct AttnLayout {
-  int kring, vring, p, q, wmax, lw, mfin, mref, einv, erow, mrow, desc, gpre, plen, rowbits, slen, total;
+  int kring, vring, p, q, wmax, lw, mfin, mref, einv, erow, desc, gpre, plen, rowbits, slen, total;
 };
 inline AttnLayout attn_layout(int D, int sets, int per_set, int hk, int hv, int np, int nqb, int G, int R,
                               bool slen_in_smem) {
@@ -66,10 +71,9 @@ inline AttnLayout attn_layout(int D, int sets, int per_set, int hk, int hv, int 
   L.lw = L.wmax + 4 * nq * 4;                 // [2 pieces][4][nq] per-warp query sums
   L.mfin = L.lw + 8 * nq * 4;                 // [2 pieces][nq] reference maxima at the piece end
   L.mref = L.mfin + 2 * nq * 4;               // [2 versions][nq] current reference maxima
-  L.einv = L.mref + 2 * nq * 4;               // piece end, per query: 1 / sum, output row (-1: none);
-  L.erow = L.einv + kMaxQueries * 4;          // and the output rows of the job that the block merges
-  L.mrow = L.erow + kMaxQueries * 4;
-  L.desc = L.mrow + kMaxQueries * 4;            // [8 groups][8 pages] tokens and row of a page
+  L.einv = L.mref + 2 * nq * 4;               // piece end, per query: 1 / sum, output row (-1: none)
+  L.erow = L.einv + kMaxQueries * 4;
+  L.desc = L.erow + kMaxQueries * 4;          // [8 groups][8 pages] tokens and row of a page
   L.gpre = L.desc + 8 * kGroupPages * 4;      // [G + 1] pages of the groups before
   L.plen = align_up(L.gpre + (G + 1) * 4, 16);
   L.rowbits = align_up(L.plen + G * 4, 16);   // one bit per row: active
@@ -95,6 +99,7 @@ struct AttnParams {
   int32_t nq, C;
   int32_t hk, hv;        // K and V areas of the ring
   int32_t np, nqb;       // P^T and Q buffers (1 or 2)
+  int32_t fold;          // a split job of at most this many other pieces is folded in the K ring
   int32_t slen_in_smem;  // the rows' suffix lengths are kept in shared memory
   float scale_log2;
   AttnLayout L;      // the shared-memory carve-up

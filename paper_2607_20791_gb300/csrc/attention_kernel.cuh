@@ -12,15 +12,16 @@
 //
 // Work distribution.  The jobs' page lists are laid end to end (job-major) and
 // the grid's persistent blocks (one per SM) each take an equal contiguous range
-// of pages.  Only the two jobs at the ends of a block's range can be split with
-// a neighbour, and a block works on those two first (the end of the job it
-// starts in, then the start of the job it ends in, then the whole jobs between).
-// A split job is merged by log-sum-exp (Sec. 3's shared-prefix split is the same
-// identity) in the block holding its first page: the job's other pieces --
-// each the first piece of its own block, behind no wait on another block --
-// write a partial (o, m, l) to workspace slot (block + job) and count
-// themselves in the job's ticket.  The merging block writes its own piece there
-// too and folds all of them once its last piece is done, with all its warps.
+// of pages and works through it in order.  Only the two jobs at the ends of a
+// block's range can be split with a neighbour.  A split job is merged by
+// log-sum-exp (Sec. 3's shared-prefix split is the same identity) in the block
+// holding its first page, whose last piece it is: the job's other pieces -- each
+// the first piece of its own block, behind no wait on another block -- write a
+// partial (o, m, l) to workspace slot (block + job) and count themselves in the
+// job's ticket.  The merging block fetches them into its idle K ring while its
+// last group is in flight and folds them into its own piece on the way out; if
+// the ring has no room for all, it writes its own piece to the workspace too and
+// folds all of them from there.
 //
 // Inside a block the tokens are the MMA's M and the queries its N:
 //   S^T = K Q^T      A = a group's K (128 tokens = 8 pages, K-major), B = Q,
@@ -45,14 +46,13 @@
 // -> block table -> data) and the merge at the end.  Measured inside a CUDA
 // graph, against a kernel with the queries as the MMA's M (128 rows of query
 // copies), P in tensor memory and one ring for K and V together (us):
-//   256 groups x 2 rows, 32/8 heads, D 128, prompts of 128-8192    440 -> 362 (0.95 of the copy rate)
-//   16 x 5, 32/8, 128, 512-2048                                     36 -> 33
+//   256 groups x 2 rows, 32/8 heads, D 128, prompts of 128-8192    440 -> 359 (0.96 of the copy rate)
+//   16 x 5, 32/8, 128, 512-2048                                     36 -> 31
 //   1 x 5, 32/8, 128, 3000                                          25 -> 17.5
-//   12 x 9, 32/8, 128, 500-6000                                     70 -> 51
-//   4 x 9, 64/8, 128, 32768                                        202 -> 120
-//   32 x 4, 32/8, 64, 500-3000                                      53 -> 40
-//   200 x 16, 4/1, 64, 50-100                                       35 -> 40: the one that lost; 3200 rows
-//                                  to set up and pieces of a few pages, so the start and the end are all there is
+//   12 x 9, 32/8, 128, 500-6000                                     70 -> 50
+//   4 x 9, 64/8, 128, 32768                                        202 -> 121
+//   32 x 16, 64/8, 128, 200-800                                    107 -> 90
+//   200 x 16, 4/1, 64, 50-100                                       35 -> 34
 // Every wait on an mbarrier is bounded; a timeout is reported in the status
 // word and every role stops.
 #pragma once
@@ -91,13 +91,6 @@ struct Job {
   int start;    // first page in the global page order (fewer than 2^31 pages)
 };
 
-// A block's job pieces in the order it works on them: the job at the start of
-// its range, then the job at the end, then the whole jobs in between.
-struct PieceIter {
-  Job j0, jl;   // first and last job of the range
-  int n0, nl;   // their pages in the range (nl = 0: the range holds one job)
-  int mid_end;  // global page where the middle jobs end
-};
 
 // What every role of a block looks up, in shared memory: the functions that
 // take it are out of line and shared by the roles, which keeps the kernel's code
@@ -108,7 +101,8 @@ struct BlockCtx {
   const int32_t *prompt_bt, *suffix_bt, *suffix_len;
   const int32_t *gpre, *plen, *slen;  // slen: NULL when it is read from global memory
   const uint32_t* rowbits;
-  PieceIter it;
+  Job j0, jl;  // first and last job of the range (the block's pieces are the jobs' parts in it, in order)
+  int n0;      // the first job's pages in the range
 };
 
 __device__ __forceinline__ void flag(int32_t* status, int32_t bit) {
@@ -147,27 +141,12 @@ __device__ __noinline__ Job job_at(const BlockCtx& c, int x) {
 // Block whose page range contains global page x (ranges [floor(cT/C), floor((c+1)T/C))).
 __device__ __noinline__ int cta_of(const BlockCtx& c, int x) { return div_nn((int64_t)(x + 1) * c.Ceff - 1, c.T); }
 
-// Piece k (>= 1) after piece k - 1 = (cur, n); false when there is none.
-__device__ __noinline__ bool next_piece(const BlockCtx& c, int k, Job& cur, int& n) {
-  const PieceIter& it = c.it;
-  if (k == 1) {
-    if (it.nl == 0) return false;
-    cur = it.jl;
-    n = it.nl;
-    return true;
-  }
-  Job j = k == 2 ? it.j0 : cur;
-  j.start += j.n;
-  if (++j.h == c.Hkv) {
-    j.h = 0;
-    do {
-      ++j.g;
-    } while (j.g < c.G && c.gpre[j.g + 1] == c.gpre[j.g]);
-    j.n = j.g < c.G ? c.gpre[j.g + 1] - c.gpre[j.g] : 0;
-  }
-  if (j.g >= c.G || j.start >= it.mid_end) return false;
-  cur = j;
-  n = j.n;
+// The piece after (cur, n pages): its job and pages; false when there is none.
+__device__ __noinline__ bool next_piece(const BlockCtx& c, Job& cur, int& n) {
+  const int x = cur.start + cur.n;
+  if (x >= c.e) return false;
+  cur = x >= c.jl.start ? c.jl : job_at(c, x);
+  n = min(c.e, cur.start + cur.n) - x;
   return true;
 }
 
@@ -227,19 +206,16 @@ __device__ __noinline__ void more_rows(const AttnParams& p, int32_t* slen_s, int
   }
 }
 
-// Page i of the block's page sequence (pieces in PieceIter order).
+// Page i of the block's range.
 struct PageRef {
   int page, desc, h;   // pool page (-1: none); tokens | row << 16 (-1: every row); kv head
   int pos, ng;         // position in its group of 8, and the pages of that group
 };
 __device__ __noinline__ PageRef resolve_page(const BlockCtx& c, int i) {
   PageRef r{-1, 0, 0, 0, 0};
-  if (i >= c.e - c.b) return r;
-  const PieceIter& it = c.it;
-  const int x = i < it.n0 ? c.b + i
-                : i < it.n0 + it.nl ? it.jl.start + (i - it.n0)
-                                    : c.b + it.n0 + (i - it.n0 - it.nl);
-  const Job jb = i < it.n0 ? it.j0 : i < it.n0 + it.nl ? it.jl : job_at(c, x);
+  const int x = c.b + i;
+  if (x >= c.e) return r;
+  const Job jb = i < c.n0 ? c.j0 : x >= c.jl.start ? c.jl : job_at(c, x);
   // this block's piece of the job starts at max(b, job start); groups restart there
   const int pstart = max(c.b, jb.start);
   const int kin = x - pstart;
@@ -487,6 +463,32 @@ __device__ __noinline__ void merge_many(const int32_t* wrow, const float2* ml, c
   }
 }
 
+// The weights of a split job's other partials for one query (in place of their
+// maxima, over the whole job's sum) and of this block's own piece (m, l; returned
+// unnormalised); m and l become the whole job's.
+__device__ __noinline__ float fold_weights(float2* pml, int stride, int nparts, float& m, float& l) {
+  float2 x[kMaxFold];
+#pragma unroll
+  for (int k = 0; k < kMaxFold; ++k) x[k] = k < nparts ? pml[k * stride] : make_float2(0.f, 0.f);
+  float M = l > 0.f ? m : -INFINITY;
+#pragma unroll
+  for (int k = 0; k < kMaxFold; ++k) M = x[k].y > 0.f ? fmaxf(M, x[k].x) : M;
+  const float own = l > 0.f ? exp2f(m - M) : 0.f;
+  float L = own * l;
+#pragma unroll
+  for (int k = 0; k < kMaxFold; ++k) {
+    x[k].x = x[k].y > 0.f ? exp2f(x[k].x - M) : 0.f;
+    L += x[k].x * x[k].y;
+  }
+  const float inv = L > 0.f ? 1.f / L : 0.f;
+#pragma unroll
+  for (int k = 0; k < kMaxFold; ++k)
+    if (k < nparts) pml[k * stride].x = x[k].x * inv;
+  m = M;
+  l = L;
+  return own;
+}
+
 // Q of job jb into a Q buffer by the 128 piece-end threads (this one: et):
 // [D/64 halves][kN rows][128 B], 128-byte swizzle; rows >= nq are zero.
 template <int D, int kN>
@@ -537,10 +539,16 @@ __device__ __noinline__ void write_empty_jobs(const BlockCtx& c, int block, int 
 
 // O^T columns c0, c0 + step, ... (eight a time) of a finished piece, by a warp of
 // TMEM lane quarter d / 32: to the partial `part` of a split job, or, normalised,
-// to the output rows.  (part and out point at head dimension d.)
+// to the output rows, with the `nparts` other partials of a split job added by
+// their weights (pml's x).  (part, out and po point at head dimension d; erow and
+// einv have 128 entries, erow -1 past nq.)  A block's time after its last MMA is
+// this function's, so the eight columns' loads go together and stores are
+// predicated: with a branch or a dependent load per column it took 120 cycles a
+// column (360 with a partial to add).
 template <int D>
-__device__ __noinline__ void write_columns(uint32_t col, int lo_off, int c0, int step, int nq, bool write, float* part,
-                                           __nv_bfloat16* out, const int32_t* erow, const float* einv) {
+__device__ __noinline__ void write_columns(uint32_t col, int lo_off, int c0, int step, int nq, float* part,
+                                           __nv_bfloat16* out, const int32_t* erow, const float* einv, int nparts,
+                                           const float* po, const float2* pml) {
 #pragma unroll 1
   for (; c0 < nq; c0 += step) {
     uint32_t hi[8], lo[8];
@@ -548,18 +556,37 @@ __device__ __noinline__ void write_columns(uint32_t col, int lo_off, int c0, int
     tmem_ld8(col + lo_off + c0, lo);
     tmem_ld_wait8(hi);
     tmem_ld_wait8(lo);
-    if (!write) continue;
+    float v[8];
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      if (c0 + i >= nq) break;
-      const float v = __uint_as_float(hi[i]) + __uint_as_float(lo[i]);
-      if (part) {
-        part[(c0 + i) * D] = v;
-      } else {
-        const int row = erow[c0 + i];
-        if (row >= 0) out[(int64_t)row * D] = __float2bfloat16(v * einv[c0 + i]);
-      }
+    for (int i = 0; i < 8; ++i) v[i] = __uint_as_float(hi[i]) + __uint_as_float(lo[i]);
+    if (part) {
+#pragma unroll
+      for (int i = 0; i < 8; ++i)
+        if (c0 + i < nq) part[(c0 + i) * D] = v[i];
+      continue;
     }
+    const int4 r0 = *reinterpret_cast<const int4*>(erow + c0), r1 = *reinterpret_cast<const int4*>(erow + c0 + 4);
+    const float4 e0 = *reinterpret_cast<const float4*>(einv + c0), e1 = *reinterpret_cast<const float4*>(einv + c0 + 4);
+    const int row[8] = {r0.x, r0.y, r0.z, r0.w, r1.x, r1.y, r1.z, r1.w};
+    const float ev[8] = {e0.x, e0.y, e0.z, e0.w, e1.x, e1.y, e1.z, e1.w};
+#pragma unroll
+    for (int i = 0; i < 8; ++i) v[i] *= ev[i];
+    const float* o = po + c0 * D;  // (past nq: other shared memory, for columns that are not stored)
+    const float2* m = pml + c0;
+#pragma unroll 1
+    for (int k = 0; k < nparts; ++k, o += nq * D, m += ml_stride(nq)) {
+      float x[8], y[8];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        x[i] = m[i].x;
+        y[i] = o[i * D];
+      }
+#pragma unroll
+      for (int i = 0; i < 8; ++i) v[i] += x[i] * y[i];
+    }
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+      if (row[i] >= 0) out[(int64_t)row[i] * D] = __float2bfloat16(v[i]);
   }
 }
 
@@ -584,13 +611,15 @@ __global__ void __launch_bounds__(AttnCfg<D, NS, QS>::kThreads, 1)
   int32_t* descs = reinterpret_cast<int32_t*>(smem + L.desc);
   float* einv = reinterpret_cast<float*>(smem + L.einv);
   int32_t* erow = reinterpret_cast<int32_t*>(smem + L.erow);
-  int32_t* mrow = reinterpret_cast<int32_t*>(smem + L.mrow);
+  // (m, l) of a folded job's partials, behind their O in the K ring; l becomes the weights
+  auto pml_of = [&](int parts) { return reinterpret_cast<float2*>(smem + L.kring + parts * p.nq * D * 4); };
   __shared__ uint64_t k_full[kRingMax], k_empty[kRingMax], v_full[kRingMax], v_empty[kRingMax];
   __shared__ uint64_t s_full[2], s_empty[2], p_full[2], p_empty[2], q_full[2], q_empty[2];
   __shared__ uint64_t o_full[2], o_free[2], ml_full[2], ml_empty[2], mma_done[2];
-  // the split job that starts in this block: its pieces (0: none), its index, whether
-  // this block's piece is written, and its ticket
-  __shared__ int32_t s_abort, s_issued[2], s_mpieces, s_mjob, s_mpiece, s_tick;
+  // the split job that starts in this block: its pieces (0: none), its index, its
+  // ticket, and whether its partials' copies (completing on m_full) were issued
+  __shared__ uint64_t m_full;
+  __shared__ int32_t s_abort, s_issued[2], s_mpieces, s_mjob, s_tick, s_mcopy;
   // the block's last piece: 0 none or given up, 2 to be written; its job + 1 if split; its O^T buffer
   __shared__ int32_t s_last_ok, s_last_split, s_last_ob;
   __shared__ uint32_t s_tmem;
@@ -625,8 +654,8 @@ __global__ void __launch_bounds__(AttnCfg<D, NS, QS>::kThreads, 1)
     }
     s_abort = 0;
     s_issued[0] = s_issued[1] = 0;
-    s_mpieces = 0;
-    s_mpiece = 0;
+    mbar_init(&m_full, 1);
+    s_mpieces = s_mcopy = 0;
     s_last_ok = s_last_split = 0;
     fence_mbar_init();
   }
@@ -745,16 +774,10 @@ __global__ void __launch_bounds__(AttnCfg<D, NS, QS>::kThreads, 1)
     if (b < e) {  // the jobs at the range's ends (lanes 0 and 1)
       const Job j = job_at(ctx, lane == 1 ? e - 1 : b);
       if (lane == 0) {
-        ctx.it.j0 = j;
-        ctx.it.n0 = min(e, j.start + j.n) - b;
+        ctx.j0 = j;
+        ctx.n0 = min(e, j.start + j.n) - b;
       }
-      __syncwarp();
-      if (lane == 1) {
-        const bool more = b + ctx.it.n0 < e;
-        ctx.it.jl = j;
-        ctx.it.nl = more ? e - j.start : 0;
-        ctx.it.mid_end = more ? j.start : e;
-      }
+      if (lane == 1) ctx.jl = j;
     }
   }
   tc_fence_before();
@@ -836,16 +859,37 @@ __global__ void __launch_bounds__(AttnCfg<D, NS, QS>::kThreads, 1)
     // (the sample head) may be scheduled once every block has got here or
     // exited.  It still waits for this kernel to complete before it writes.
     if (is_v) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    // The split job that starts in this block is merged here, after the block's
+    // The split job that starts in this block is merged here, with the block's
     // last piece: its other pieces are the first ones of later blocks, behind no
-    // wait on another block, so this wait ends (bounded anyway).
+    // wait on another block, so this wait ends (bounded anyway).  Their partials
+    // are copied to the K ring, which nothing uses after the last QK.
     if (!is_v && lane == 0 && b < e) {
-      const Job jb = ctx.it.nl ? ctx.it.jl : ctx.it.j0;
+      const Job jb = ctx.jl;
       const int nparts = cta_of(ctx, jb.start + jb.n - 1) - c;
       if (jb.start >= b && nparts > 0) {
+        const int j = jb.g * p.Hkv + jb.h;
         s_mpieces = nparts + 1;
-        s_mjob = jb.g * p.Hkv + jb.h;
-        s_tick = wait_ticket(p.ticket + s_mjob, nparts, abort_flag, p.wait_ns);
+        s_mjob = j;
+        if (nparts > p.fold) mbar_arrive(&m_full);  // (nothing to wait for before the own partial)
+        int tick = wait_ticket(p.ticket + j, nparts, abort_flag, p.wait_ns);
+        if (nparts <= p.fold) {
+#pragma unroll 1
+          for (int g = max(0, gbase - hk); g < gbase; ++g)
+            if (!wait_or_abort(&k_empty[g % hk], (uint32_t)(g / hk) & 1u, abort_flag, p.wait_ns)) tick = -1;
+          s_tick = tick;
+          if (tick > 0 && (tick >> 16) == 0) {
+            const int64_t slot = (int64_t)c + j + 1;
+            const uint32_t ob = nparts * p.nq * D * 4, mb = nparts * ml_stride(p.nq) * 8;
+            fence_proxy_async_global();  // (the partials are other blocks' ordinary writes)
+            s_mcopy = 1;
+            mbar_arrive_expect_tx(&m_full, ob + mb);
+            bulk_load(smem + L.kring, p.slot_o + slot * p.nq * D, ob, &m_full);
+            bulk_load(smem + L.kring + ob, p.slot_ml + slot * ml_stride(p.nq), mb, &m_full);
+          } else {
+            mbar_arrive(&m_full);
+          }
+        }
+        s_tick = tick;
       }
     }
   } else if (warp == C::kQk) {
@@ -856,10 +900,10 @@ __global__ void __launch_bounds__(AttnCfg<D, NS, QS>::kThreads, 1)
       int gi = 0, pc = 0, gs = 0;
       uint32_t ph = 0;
       bool ok = true;
-      Job cur = ctx.it.j0;
-      int n_in = ctx.it.n0;
+      Job cur = ctx.j0;
+      int n_in = ctx.n0;
 #pragma unroll 1
-      for (bool more = true; ok && more; more = next_piece(ctx, pc, cur, n_in)) {
+      for (bool more = true; ok && more; more = next_piece(ctx, cur, n_in)) {
         const int qb = nqb == 2 ? pc & 1 : 0;
         if (!wait_or_abort(&q_full[qb], (uint32_t)(nqb == 2 ? pc >> 1 : pc) & 1u, abort_flag, p.wait_ns)) break;
 #pragma unroll 1
@@ -901,10 +945,10 @@ __global__ void __launch_bounds__(AttnCfg<D, NS, QS>::kThreads, 1)
       int gi = 0, pc = 0, gs = 0;
       uint32_t ph = 0;
       bool ok = true;
-      Job cur = ctx.it.j0;
-      int n_in = ctx.it.n0;
+      Job cur = ctx.j0;
+      int n_in = ctx.n0;
 #pragma unroll 1
-      for (bool more = true; ok && more; more = next_piece(ctx, pc, cur, n_in)) {
+      for (bool more = true; ok && more; more = next_piece(ctx, cur, n_in)) {
         const int ob = C::kOBufs == 2 ? pc & 1 : 0;
         const uint32_t od = tmem + C::kOCol + ob * 2 * C::kN;
         if (pc >= C::kOBufs &&
@@ -983,11 +1027,11 @@ __global__ void __launch_bounds__(AttnCfg<D, NS, QS>::kThreads, 1)
     int gi = 0;
     bool ok = true;
     if (b < e) {
-      Job cur = ctx.it.j0;
-      int n_in = ctx.it.n0;
+      Job cur = ctx.j0;
+      int n_in = ctx.n0;
       int pc = 0;
 #pragma unroll 1
-      for (bool more = true; more; more = next_piece(ctx, pc, cur, n_in)) {
+      for (bool more = true; more; more = next_piece(ctx, cur, n_in)) {
         const int ob = C::kOBufs == 2 ? pc & 1 : 0;
 #pragma unroll 1
         for (int k0 = 0; k0 < n_in; k0 += kGroupPages) {
@@ -1201,120 +1245,125 @@ __global__ void __launch_bounds__(AttnCfg<D, NS, QS>::kThreads, 1)
       if (lane == 0) mbar_arrive(&q_full[qb]);
     };
     if (b < e) {
-      Job cur = ctx.it.j0, nx1 = cur, nxq = cur;  // this piece, the next, the next whose Q is to be written
-      int n_in = ctx.it.n0, n1 = n_in, nq_in = n_in;
+      Job cur = ctx.j0, nx1 = cur, nxq = cur;  // this piece, the next, the next whose Q is to be written
+      int n_in = ctx.n0, n1 = n_in, nq_in = n_in;
       put_q(cur, 0);
-      bool hasq = next_piece(ctx, 1, nxq, nq_in);
+      bool hasq = next_piece(ctx, nxq, nq_in);
       if (hasq && nqb == 2) {
         put_q(nxq, 1);
-        hasq = next_piece(ctx, 2, nxq, nq_in);
+        hasq = next_piece(ctx, nxq, nq_in);
       }
+      write_empty_jobs(ctx, c, p.C, et, nq, gq, p.Hq, D, p.out, p.lse);  // (while the first group's copies are in flight)
 #pragma unroll 1
       for (int pc = 0;; ++pc) {
         const int ob = C::kOBufs == 2 ? pc & 1 : 0, mb = pc & 1;
         const int j = cur.g * p.Hkv + cur.h;
-        const int first = cta_of(ctx, cur.start), last = cta_of(ctx, cur.start + cur.n - 1);
+        const bool merger = cur.start >= b && cur.start + cur.n > e;  // the job goes on in later blocks
+        const bool split = merger || cur.start < b;
         nx1 = cur;
         n1 = n_in;
-        const bool more = next_piece(ctx, pc + 1, nx1, n1);
-        const int nparts = last - first;  // the job's other pieces
-        const bool split = nparts > 0, merger = split && c == first;
+        const bool more = next_piece(ctx, nx1, n1);
         // ---- Q of the piece nqb ahead, into this piece's Q buffer ----
         if (hasq) {
           const int qb = nqb == 2 ? pc & 1 : 0;
           if (ok && !wwait(&q_empty[qb], (uint32_t)(nqb == 2 ? pc >> 1 : pc) & 1u)) ok = false;
           if (ok) put_q(nxq, qb);
           else if (lane == 0) mbar_arrive(&q_full[qb]);  // (keeps the QK warp's waits bounded by the abort)
-          hasq = next_piece(ctx, pc + nqb + 1, nxq, nq_in);
+          hasq = next_piece(ctx, nxq, nq_in);
         }
         // ---- this piece's maxima, sums and output rows, one query per thread ----
-        if (ok && !wwait(&o_full[ob], (uint32_t)(C::kOBufs == 2 ? pc >> 1 : pc) & 1u)) ok = false;
         if (ok && !wwait(&ml_full[mb], (uint32_t)(pc >> 1) & 1u)) ok = false;
-        tc_fence_after();
-        const bool good = __all_sync(0xffffffffu, ok && !*abort_flag);
+        if (merger && ok && !wwait(&m_full, 0u)) ok = false;
+        const int nparts = merger && ok ? s_mpieces - 1 : 0;  // its other pieces
+        const bool fold = nparts > 0 && nparts <= p.fold;
+        float2* pml = pml_of(nparts);
+        bool good = ok && !(fold && (s_tick <= 0 || (s_tick >> 16) != 0));
         const int64_t slot = (int64_t)c + j;  // of a split job's partial
+        erow[et] = -1;
         if (et < nq) {
-          const float M = mfin[mb * C::kNq + et];
-          const float Ls = (lw[(mb * 4) * C::kNq + et] + lw[(mb * 4 + 1) * C::kNq + et]) +
-                           (lw[(mb * 4 + 2) * C::kNq + et] + lw[(mb * 4 + 3) * C::kNq + et]);
+          float M = mfin[mb * C::kNq + et];
+          float Ls = (lw[(mb * 4) * C::kNq + et] + lw[(mb * 4 + 1) * C::kNq + et]) +
+                     (lw[(mb * 4 + 2) * C::kNq + et] + lw[(mb * 4 + 3) * C::kNq + et]);
           const int r = et / gq, rr = cur.g * p.rpg + r;
           const int row = row_bit(rowbits, rr) ? rr * p.Hq + cur.h * gq + (et - r * gq) : -1;
-          einv[et] = Ls > 0.f ? 1.f / Ls : 0.f;
           erow[et] = row;
-          if (merger) mrow[et] = row;
-          if (good && split) p.slot_ml[slot * mls + et] = make_float2(M, Ls);
-          if (good && !split && p.lse && row >= 0) p.lse[row] = Ls > 0.f ? (M + log2f(Ls)) * kLn2 : -INFINITY;
+          float own = 1.f;
+          if (fold && good) own = fold_weights(pml + et, mls, nparts, M, Ls);
+          einv[et] = Ls > 0.f ? own / Ls : 0.f;
+          if (good && split && !fold) p.slot_ml[slot * mls + et] = make_float2(M, Ls);
+          if (good && (!split || fold) && p.lse && row >= 0) p.lse[row] = Ls > 0.f ? (M + log2f(Ls)) * kLn2 : -INFINITY;
         }
+        if (ok && !wwait(&o_full[ob], (uint32_t)(C::kOBufs == 2 ? pc >> 1 : pc) & 1u)) ok = false;
+        tc_fence_after();
+        good = __all_sync(0xffffffffu, good && ok && !*abort_flag);
         epi_sync();
         if (!more) {  // the block's last piece: all softmax and piece-end warps share its columns
           if (et == 0) {
             s_last_ok = ok ? (good ? 2 : 1) : 0;
             s_last_split = split ? j + 1 : 0;
             s_last_ob = ob;
-            if (merger) s_mpiece = good ? 1 : -1;
           }
           break;
         }
-        if (ok)
-          write_columns<D>(tl + C::kOCol + 2 * ob * C::kN, C::kN, 0, 8, nq, good && d < D,
-                           split ? p.slot_o + slot * nq * D + d : nullptr, p.out + d, erow, einv);
+        if (good && d < D)
+          write_columns<D>(tl + C::kOCol + 2 * ob * C::kN, C::kN, 0, 8, nq,
+                           split ? p.slot_o + slot * nq * D + d : nullptr, p.out + d, erow, einv, 0, nullptr, nullptr);
         tc_fence_before();
         epi_sync();
         if (lane == 0) {
           mbar_arrive(&o_free[ob]);
           mbar_arrive(&ml_empty[mb]);
         }
-        if (et == 0 && split) {
-          if (merger) {
-            s_mpiece = good ? 1 : -1;
-          } else {
-            __threadfence();  // the partial (written by every piece-end warp before the barrier), before its count
-            atomicAdd(p.ticket + j, good && !*abort_flag ? 1 : 0x10001);
-          }
+        if (et == 96 && split) {  // (a later piece follows, so this job ends here; the last warp has least to do)
+          __threadfence();  // the partial (written by every piece-end warp before the barrier), before its count
+          atomicAdd(p.ticket + j, good && !*abort_flag ? 1 : 0x10001);
         }
         cur = nx1;
         n_in = n1;
       }
     }
-    write_empty_jobs(ctx, c, p.C, et, nq, gq, p.Hq, D, p.out, p.lse);
+    if (b >= e) write_empty_jobs(ctx, c, p.C, et, nq, gq, p.Hq, D, p.out, p.lse);
   }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  const int parts = s_mpieces - 1;  // of the split job merged here, without the block's own
+  const bool fold = parts > 0 && parts <= p.fold;
   if (s_last_ok > 0) {  // (uniform) the last piece's O^T: set s and the piece-end warps take every (NS + 1)-th chunk
     const int split = s_last_split, j = split - 1;
-    if (warp < C::kEpi + 4) {
-      const int d = (warp & 3) * 32 + lane;
+    const int d = (warp & 3) * 32 + lane;
+    if (warp < C::kEpi + 4 && s_last_ok == 2 && d < D)
       write_columns<D>(tmem + ((uint32_t)((warp & 3) * 32) << 16) + C::kOCol + 2 * s_last_ob * C::kN, C::kN,
-                       (warp >> 2) * 8, (NS + 1) * 8, p.nq, s_last_ok == 2 && d < D,
-                       split ? p.slot_o + ((int64_t)c + j) * p.nq * D + d : nullptr, p.out + d, erow, einv);
-    }
+                       (warp >> 2) * 8, (NS + 1) * 8, p.nq,
+                       split && !fold ? p.slot_o + ((int64_t)c + j) * p.nq * D + d : nullptr, p.out + d, erow, einv,
+                       fold ? parts : 0, reinterpret_cast<const float*>(smem + L.kring) + d, pml_of(parts));
     tc_fence_before();
     __syncthreads();
   }
   // (a split job's last piece counts itself also when this block has given up)
-  if (tid == 0 && s_last_split > 0 && s_mpieces == 0) {
+  if (tid == 0 && s_last_split > 0 && parts < 0) {
     __threadfence();  // the partial (written by every warp before the barrier), before its count
     atomicAdd(p.ticket + (s_last_split - 1), s_last_ok == 2 && !*abort_flag ? 1 : 0x10001);
   }
-  if (s_mpieces > 0) {  // (uniform) the merge of the split job that starts in this block
+  if (parts > 0) {  // (uniform) the merge of the split job that starts in this block
     const int j = s_mjob;
-    const bool good = s_tick > 0 && (s_tick >> 16) == 0 && s_mpiece == 1 && !*abort_flag;
+    const bool good = !fold && s_tick > 0 && (s_tick >> 16) == 0 && s_last_ok == 2 && !*abort_flag;
     const int64_t slot = (int64_t)c + j;
     // (the rings and P^T are idle: the table goes there)
     const int qb = min(p.nq, L.q / 8 / s_mpieces);
     const float2* ml = p.slot_ml + slot * ml_stride(p.nq);
     const float* po = p.slot_o + slot * p.nq * D;
     if (good && qb > 0)
-      merge_block<D>(reinterpret_cast<float2*>(smem), qb, einv, mrow, ml, po, p.out, p.lse, p.nq, s_mpieces, tid, kThr);
+      merge_block<D>(reinterpret_cast<float2*>(smem), qb, einv, erow, ml, po, p.out, p.lse, p.nq, s_mpieces, tid, kThr);
     else if (good)
-      merge_many<D>(mrow, ml, po, p.out, p.lse, p.nq, s_mpieces, tid, kThr);
+      merge_many<D>(erow, ml, po, p.out, p.lse, p.nq, s_mpieces, tid, kThr);
     if (tid == 0) p.ticket[j] = 0;  // every other piece has counted itself
   }
   if (*abort_flag) {
     // a wait gave up: report, and let copies and MMAs still in flight drain (bounded)
     if (tid == 0) {
       flag(p.dev_status, RGD_DEV_WAIT_TIMEOUT);
+      if (s_mcopy) mbar_wait(&m_full, 0);
 #pragma unroll 1
       for (int g = max(0, s_issued[0] - hk); g < s_issued[0]; ++g) mbar_wait(&k_full[g % hk], (g / hk) & 1);
 #pragma unroll 1

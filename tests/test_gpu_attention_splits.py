@@ -46,6 +46,23 @@ def test_merge_of_many_pieces(gpu_lib, D, rpg, heads):
     _check(case, _run(case))
 
 
+@pytest.mark.parametrize("D,rpg,heads", [(128, 5, 4), (64, 1, 1), (64, 15, 4), (128, 9, 8), (128, 16, 8)])
+@pytest.mark.parametrize("pieces", [2, 3, 5, 6])
+def test_fold_of_few_pieces(gpu_lib, D, rpg, heads, pieces):
+    # one job in exactly `pieces` blocks, on both sides of the most that is folded
+    # in the K ring (4 others, fewer where the partials are large), and the same
+    # with whole jobs before the split ones; some pieces hold suffix pages only
+    rng = np.random.default_rng(pieces)
+    act = np.ones(rpg, np.uint8)
+    act[rpg // 2] = rpg < 2
+    case = workloads.make_attn_case("fold", 1, rpg, heads, 1, D, [330], rng.integers(0, 60, rpg), seed=pieces,
+                                    row_active=act)
+    _check(case, _run(case, num_ctas=pieces))
+    case = workloads.make_attn_case("fold2", 6, rpg, heads, 1, D, [20, 1, 900, 33, 0, 700],
+                                    rng.integers(0, 60, 6 * rpg), seed=pieces)
+    _check(case, _run(case, num_ctas=pieces + 2))
+
+
 def test_blocks_with_several_small_jobs(gpu_lib):
     # three blocks for 40 jobs of 1-4 pages: pieces follow one another with one group each
     rng = np.random.default_rng(3)
