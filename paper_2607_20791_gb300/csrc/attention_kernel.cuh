@@ -1385,20 +1385,9 @@ int launch_attn_cfg(const CUtensorMap& tmK, const CUtensorMap& tmV, const AttnPa
                     cudaStream_t st) {
   static bool done = false;
   if (int rc = ensure_smem(attn_kernel<D, NS, QS>, kSmemLimit, &done)) return rc;
-  // a programmatic dependent of the previous kernel on the stream: its blocks are
-  // placed, and set up what needs no input, while that kernel finishes
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(p.C);
-  cfg.blockDim = dim3(AttnCfg<D, NS, QS>::kThreads);
-  cfg.dynamicSmemBytes = smem_bytes;
-  cfg.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  cudaError_t e = cudaLaunchKernelEx(&cfg, attn_kernel<D, NS, QS>, tmK, tmV, p);
-  if (e == cudaSuccess) e = cudaGetLastError();
+  // (its blocks are placed, and set up what needs no input, while the previous kernel finishes)
+  const cudaError_t e = launch_dependent(attn_kernel<D, NS, QS>, p.C, AttnCfg<D, NS, QS>::kThreads, smem_bytes, st,
+                                         tmK, tmV, p);
   return e == cudaSuccess ? RGD_OK : cuda_error(e, "attention launch");
 }
 

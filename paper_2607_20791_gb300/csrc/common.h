@@ -21,6 +21,25 @@ inline int cuda_error(cudaError_t e, const char* what) {
 
 inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
+// Launches a kernel as a programmatic dependent of the previous kernel on the
+// stream: it is scheduled while that kernel finishes, and waits for it
+// (griddepcontrol.wait) before it reads or writes memory.
+template <typename... P, typename... A>
+cudaError_t launch_dependent(void (*kernel)(P...), int grid, int block, int smem, cudaStream_t st, A&&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)grid);
+  cfg.blockDim = dim3((unsigned)block);
+  cfg.dynamicSmemBytes = (size_t)smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+  return e == cudaSuccess ? cudaGetLastError() : e;
+}
+
 // Opts a kernel into `bytes` of dynamic shared memory once per process.
 template <typename Kernel>
 int ensure_smem(Kernel k, int bytes, bool* done) {

@@ -27,6 +27,8 @@ namespace {
 
 __global__ void gate_state_init_kernel(rgd_gate_state* st, int32_t groups) {
   const int32_t g = blockIdx.x * blockDim.x + threadIdx.x;
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");  // (a dependent waits for this kernel's end)
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   if (g >= groups) return;
   rgd_gate_state s;
   s.node = 0;
@@ -40,26 +42,106 @@ __global__ void gate_state_init_kernel(rgd_gate_state* st, int32_t groups) {
   st[g] = s;
 }
 
-__global__ void probe_gate_kernel(TrieView t, int32_t groups, int32_t rows_per_group,
-                                  const int32_t* __restrict__ tokens, int32_t n_tokens, int64_t stride,
-                                  int32_t eos, int32_t max_len, rgd_gate_state* __restrict__ state,
-                                  uint8_t* __restrict__ row_active, int32_t* dev_status) {
-  const int32_t g = blockIdx.x * blockDim.x + threadIdx.x;
+// A trie node during a warp's walk: its first edge and their number.
+struct WalkNode {
+  int32_t begin, count;
+};
+
+// The edge labelled `tok` out of node n, by a warp: 32 edges a step, so a node of
+// up to 32 children takes one load, the root of a thousand two.  {node it leads
+// to, whether that node confirms}, or {-1, 0}; n becomes that node.
+__device__ __forceinline__ int2 warp_child(const TrieView& t, WalkNode& n, int32_t tok, int lane) {
+  int32_t lo = n.begin, cnt = n.count;
+#pragma unroll 1
+  while (cnt > 32) {  // the last of 32 evenly spaced edges that is not above tok
+    const int32_t step = (cnt + 31) >> 5, i = lane * step;
+    const bool le = i < cnt && __ldg(&t.edges[lo + i].x) <= tok;
+    const int32_t k = __popc(__ballot_sync(0xffffffffu, le));
+    if (k == 0) return make_int2(-1, 0);
+    lo += (k - 1) * step;
+    cnt = min(step, cnt - (k - 1) * step);
+  }
+  int4 e = make_int4(-1, -1, 0, 0);
+  if (lane < cnt) e = __ldg(t.edges + lo + lane);
+  const uint32_t hit = __ballot_sync(0xffffffffu, lane < cnt && e.x == tok);
+  if (hit == 0) return make_int2(-1, 0);
+  const int src = __ffs(hit) - 1;
+  n.begin = __shfl_sync(0xffffffffu, e.z, src);
+  const int32_t w = __shfl_sync(0xffffffffu, e.w, src);
+  n.count = w & 0x7fffffff;
+  return make_int2(__shfl_sync(0xffffffffu, e.y, src), w < 0 ? 1 : 0);
+}
+
+// One warp per group.  The walk is a chain of dependent loads, an L2 round trip
+// each, and nothing else: so the tokens come 32 at a time, a token takes one
+// round trip (two or three out of a large node), and the state and the rows' mask
+// are the lanes' together.  Every lane holds the same gate state.  Inside a graph:
+// 1024 probes of 32 tokens against 1000 prefixes 14.5 us with a thread a group and
+// a binary search over separate arrays, 6.4 so; 4096 of 64 tokens against 2000:
+// 20 us, 7.7; one probe of 32 tokens: 7.5 us, 2.6.
+constexpr int kGateThreads = 128;
+__global__ void __launch_bounds__(kGateThreads)
+    probe_gate_kernel(TrieView t, int32_t groups, int32_t rows_per_group, const int32_t* __restrict__ tokens,
+                      int32_t n_tokens, int64_t stride, int32_t eos, int32_t max_len,
+                      rgd_gate_state* __restrict__ state, uint8_t* __restrict__ row_active, int32_t* dev_status) {
+  const int lane = threadIdx.x & 31;
+  const int32_t g = blockIdx.x * (kGateThreads / 32) + (int)(threadIdx.x >> 5);
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");  // (a dependent waits for this kernel's end)
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   if (g >= groups) return;
+  const bool root_has_children = __ldg(t.child_begin + 1) > 0;
+  const int32_t* toks = tokens + (int64_t)g * stride;
+  int32_t mine = lane < n_tokens ? __ldg(toks + lane) : 0;
   rgd_gate_state s = state[g];
-  const bool root_has_children = __ldg(t.child_begin + 1) > __ldg(t.child_begin);
+  WalkNode n{0, 0};
+  if (!s.done && !s.confirmed) {
+    n.begin = __ldg(t.child_begin + s.node);
+    n.count = __ldg(t.child_begin + s.node + 1) - n.begin;
+  }
   bool bad_token = false;
+#pragma unroll 1
   for (int32_t k = 0; k < n_tokens && !s.done; ++k) {
-    const int32_t y = __ldg(tokens + (int64_t)g * stride + k);
+    const int32_t at = k & 31;
+    if (k > 0 && at == 0) mine = k + lane < n_tokens ? __ldg(toks + k + lane) : 0;
+    if (s.confirmed) {
+      // every further token only counts, up to the stop token or the one that
+      // reaches max_len: all of the chunk's before that at once
+      const bool in = lane >= at && k - at + lane < n_tokens;
+      const bool stop = eos >= 0 && mine == eos;
+      const uint32_t good = __ballot_sync(0xffffffffu, in && !stop && mine >= 0);
+      const bool last = ((good >> lane) & 1u) != 0 &&
+                        __popc(good & (0xffffffffu >> (31 - lane))) == max(1, max_len - s.length);
+      const uint32_t end = __ballot_sync(0xffffffffu, in && (stop || last));
+      const uint32_t bad = __ballot_sync(0xffffffffu, in && !stop && mine < 0);
+      const int n_chunk = end ? __ffs(end) - 1 : 32;  // (chunk position of the token that ends the probe)
+      const uint32_t before = n_chunk == 32 ? 0xffffffffu : (1u << n_chunk) - 1u;
+      const int counted = __popc(good & before);
+      s.steps += counted;
+      s.length += counted;
+      bad_token = bad_token || (bad & before) != 0;
+      k += n_chunk - at;
+      if (n_chunk == 32) {
+        --k;  // (the next chunk's first token)
+        continue;
+      }
+    }
+    const int32_t y = __shfl_sync(0xffffffffu, mine, k & 31);
     if (y < 0 && !(eos >= 0 && y == eos)) {
       bad_token = true;
       continue;
     }
-    consume_token(t, s, y, eos, max_len, root_has_children);
+    consume_token_with(s, y, eos, max_len, root_has_children,
+                       [&](int32_t tok) { return warp_child(t, n, tok, lane); });
   }
-  state[g] = s;
-  if (bad_token && dev_status) atomicOr(dev_status, RGD_DEV_BAD_TOKEN);
-  mask_rows(s, row_active, g, rows_per_group);
+  if (lane == 0) {
+    state[g] = s;
+    if (bad_token && dev_status) atomicOr(dev_status, RGD_DEV_BAD_TOKEN);
+  }
+  if (!row_active) return;
+  uint8_t* ra = row_active + (int64_t)g * rows_per_group;
+  if (s.done && lane == 0) ra[0] = 0;
+  if (s.decision == RGD_REFUSAL)
+    for (int32_t i = 1 + lane; i < rows_per_group; i += 32) ra[i] = 0;
 }
 
 // ---------------------------------------------------------------------------
@@ -338,11 +420,11 @@ __global__ void __cluster_dims__(kSoftCluster, 1, 1) __launch_bounds__(kSoftThre
     for (int32_t k = tid; k < nslot; k += kSoftThreads) {
       int32_t a = eos;
       if (k < nc) {
-        a = __ldg(t.child_tok + cb + k);
-        const int32_t nd = __ldg(t.child_node + cb + k);
+        const int4 e = __ldg(t.edges + cb + k);
+        a = e.x;
         sh.slot_tok[k] = a;
-        sh.slot_node[k] = nd;
-        sh.slot_conf[k] = __ldg(t.confirm + nd);
+        sh.slot_node[k] = e.y;
+        sh.slot_conf[k] = e.w < 0 ? 1 : 0;
       }
       if (maybe_soft) {
         const bool ok = a >= 0 && a < vocab && (k == nc || a != eos);
@@ -641,23 +723,20 @@ extern "C" int rgd_trie_create(const int32_t* tokens, const int64_t* offsets, in
     terminal[node] = 1;
   }
   const int32_t nn = (int32_t)kids.size();
-  std::vector<int32_t> begin(nn + 1, 0), ctok, cnode;
-  std::vector<uint8_t> confirm(nn, 0);
+  std::vector<int32_t> begin(nn + 1, 0);
   int32_t max_children = 0;
   for (int32_t n = 0; n < nn; ++n) {
     max_children = std::max(max_children, (int32_t)kids[n].size());
-    begin[n] = (int32_t)ctok.size();
-    for (const auto& kv : kids[n]) {
-      ctok.push_back(kv.first);
-      cnode.push_back(kv.second);
+    begin[n + 1] = begin[n] + (int32_t)kids[n].size();
+  }
+  std::vector<int4> edges;
+  for (int32_t n = 0; n < nn; ++n) {
+    for (const auto& [tok, node] : kids[n]) {
+      const uint32_t confirm = terminal[node] && depth[node] >= min_confirm ? 1u << 31 : 0u;
+      edges.push_back(make_int4(tok, node, begin[node], (int32_t)((uint32_t)kids[node].size() | confirm)));
     }
-    confirm[n] = (terminal[n] && depth[n] >= min_confirm) ? 1 : 0;
   }
-  begin[nn] = (int32_t)ctok.size();
-  if (ctok.empty()) {  // keep device arrays non-empty
-    ctok.push_back(-1);
-    cnode.push_back(0);
-  }
+  if (edges.empty()) edges.push_back(make_int4(-1, 0, 0, 0));  // keep the device array non-empty
   rgd_trie* t = new rgd_trie();
   t->num_nodes = nn;
   t->num_edges = begin[nn];
@@ -670,9 +749,7 @@ extern "C" int rgd_trie_create(const int32_t* tokens, const int64_t* offsets, in
     if (err == cudaSuccess) err = cudaMemcpy(*dst, src, bytes, cudaMemcpyHostToDevice);
   };
   upload((void**)&t->child_begin, begin.data(), begin.size() * sizeof(int32_t));
-  upload((void**)&t->child_tok, ctok.data(), ctok.size() * sizeof(int32_t));
-  upload((void**)&t->child_node, cnode.data(), cnode.size() * sizeof(int32_t));
-  upload((void**)&t->confirm, confirm.data(), confirm.size());
+  upload((void**)&t->edges, edges.data(), edges.size() * sizeof(int4));
   if (err != cudaSuccess) {
     rgd_trie_destroy(t);
     return cuda_error(err, "rgd_trie_create upload");
@@ -684,9 +761,7 @@ extern "C" int rgd_trie_create(const int32_t* tokens, const int64_t* offsets, in
 extern "C" int rgd_trie_destroy(rgd_trie* t) {
   if (!t) return RGD_OK;
   cudaFree(t->child_begin);
-  cudaFree(t->child_tok);
-  cudaFree(t->child_node);
-  cudaFree(t->confirm);
+  cudaFree(t->edges);
   delete t;
   return RGD_OK;
 }
@@ -705,8 +780,8 @@ extern "C" int rgd_gate_state_init(rgd_gate_state* state, int32_t groups, rgd_st
   if (groups == 0) return RGD_OK;
   RGD_CHECK_ARG(state != nullptr, "rgd_gate_state_init: state is NULL");
   const int threads = 128;
-  gate_state_init_kernel<<<(groups + threads - 1) / threads, threads, 0, (cudaStream_t)stream>>>(state, groups);
-  cudaError_t e = cudaGetLastError();
+  const cudaError_t e = launch_dependent(gate_state_init_kernel, (groups + threads - 1) / threads, threads, 0,
+                                         (cudaStream_t)stream, state, groups);
   return e == cudaSuccess ? RGD_OK : cuda_error(e, "gate_state_init launch");
 }
 
@@ -721,12 +796,11 @@ extern "C" int rgd_probe_gate(const rgd_trie* trie, int32_t groups, int32_t rows
   RGD_CHECK_ARG(max_len >= 1, "rgd_probe_gate: max_len must be >= 1");
   if (groups == 0 || n_tokens == 0) return RGD_OK;
   RGD_CHECK_ARG(probe_tokens != nullptr && state != nullptr, "rgd_probe_gate: tokens/state NULL");
-  TrieView v{trie->child_begin, trie->child_tok, trie->child_node, trie->confirm};
-  const int threads = 128;
-  probe_gate_kernel<<<(groups + threads - 1) / threads, threads, 0, (cudaStream_t)stream>>>(
-      v, groups, rows_per_group, probe_tokens, n_tokens, token_stride, eos_token, max_len, state, row_active,
-      dev_status);
-  cudaError_t e = cudaGetLastError();
+  TrieView v{trie->child_begin, trie->edges};
+  constexpr int kPer = kGateThreads / 32;  // groups per block
+  const cudaError_t e = launch_dependent(probe_gate_kernel, groups / kPer + (groups % kPer != 0), kGateThreads, 0,
+                                         (cudaStream_t)stream, v, groups, rows_per_group, probe_tokens, n_tokens,
+                                         token_stride, eos_token, max_len, state, row_active, dev_status);
   return e == cudaSuccess ? RGD_OK : cuda_error(e, "probe_gate launch");
 }
 
@@ -749,7 +823,7 @@ extern "C" int rgd_soft_gate(const rgd_trie* trie, int32_t groups, int32_t rows_
   if (groups == 0) return RGD_OK;
   RGD_CHECK_ARG(probe_logits != nullptr && state != nullptr && token_out != nullptr,
                 "rgd_soft_gate: logits/state/token_out NULL");
-  TrieView tv{trie->child_begin, trie->child_tok, trie->child_node, trie->confirm};
+  TrieView tv{trie->child_begin, trie->edges};
   cudaStream_t st = (cudaStream_t)stream;
   const int es = dtype == RGD_F32 ? 4 : 2;
   const bool vec = aligned16(probe_logits) && (row_stride * es) % 16 == 0;  // 16-byte vector loads

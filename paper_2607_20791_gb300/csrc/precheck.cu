@@ -5,10 +5,12 @@
 // its probe row is masked, so only its sample rows decode.
 //
 // One block per group: each thread reads a strided share of the group's d
-// activations (consecutive threads, consecutive elements: coalesced), keeps an
-// fp32 partial dot product, and the block reduces them (warp shuffles, then
-// shared memory).  The readout is d + 1 parameters, so the kernel is a
-// launch-latency-bound GEMV.
+// activations (consecutive threads, consecutive 16-byte vectors or, where a row
+// does not start on 16 bytes, elements: coalesced), keeps an fp32 partial dot
+// product, and the block reduces them (warp shuffles, then shared memory).  At a
+// few prompts a launch is all it costs (1.9 us inside a graph, 1.3 as a
+// programmatic dependent); a batch is a read of the activations: 4096 prompts of
+// 8192 bf16 took 17.1 us by elements, 14.4 by vectors.
 #include <cuda_bf16.h>
 
 #include <cmath>
@@ -31,18 +33,53 @@ __device__ __forceinline__ float load_act<uint16_t>(const uint16_t* p, int64_t i
   return __uint_as_float((uint32_t)__ldg(p + i) << 16);  // bf16 widened exactly
 }
 
+// Element e of a 16-byte vector of activations.
+template <typename T>
+__device__ __forceinline__ float vec_act(const uint4& x, int e);
+template <>
+__device__ __forceinline__ float vec_act<float>(const uint4& x, int e) {
+  return __uint_as_float(e == 0 ? x.x : e == 1 ? x.y : e == 2 ? x.z : x.w);
+}
+template <>
+__device__ __forceinline__ float vec_act<uint16_t>(const uint4& x, int e) {
+  const uint32_t u = (e >> 1) == 0 ? x.x : (e >> 1) == 1 ? x.y : (e >> 1) == 2 ? x.z : x.w;
+  return __uint_as_float((e & 1) ? (u & 0xffff0000u) : (u << 16));
+}
+
 template <typename T>
 __global__ void __launch_bounds__(kPrecheckThreads)
-    precheck_kernel(int32_t d, const T* __restrict__ h, const float* __restrict__ w, float bias, float theta,
+    precheck_kernel(int32_t d, bool vec, const T* __restrict__ h, const float* __restrict__ w, float bias, float theta,
                     int32_t rows_per_group, float* prob_out, rgd_gate_state* state, uint8_t* row_active) {
   __shared__ float part[kPrecheckThreads / 32];
   const int g = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const T* hg = h + (int64_t)g * d;
   float acc = 0.f;
-  // (unrolled so that a thread's loads are all in flight together; the sums
-  // stay in index order)
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");  // (a dependent waits for this kernel's end)
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  if (vec) {
+    constexpr int E = 16 / (int)sizeof(T);
+    const uint4* hv = reinterpret_cast<const uint4*>(hg);
+    const float4* wv = reinterpret_cast<const float4*>(w);
+    float4 sum = make_float4(0.f, 0.f, 0.f, 0.f);  // (four short sums round less than a long one)
+#pragma unroll 4
+    for (int i = tid; i < d / E; i += kPrecheckThreads) {
+      const uint4 x = __ldg(hv + i);
+#pragma unroll
+      for (int q = 0; q < E / 4; ++q) {
+        const float4 y = __ldg(wv + i * (E / 4) + q);
+        sum.x = fmaf(y.x, vec_act<T>(x, 4 * q), sum.x);
+        sum.y = fmaf(y.y, vec_act<T>(x, 4 * q + 1), sum.y);
+        sum.z = fmaf(y.z, vec_act<T>(x, 4 * q + 2), sum.z);
+        sum.w = fmaf(y.w, vec_act<T>(x, 4 * q + 3), sum.w);
+      }
+    }
+    acc = (sum.x + sum.y) + (sum.z + sum.w);
+  } else {
+    // (unrolled so that a thread's loads are all in flight together; the sums
+    // stay in index order)
 #pragma unroll 16
-  for (int i = tid; i < d; i += kPrecheckThreads) acc = fmaf(__ldg(w + i), load_act<T>(hg, i), acc);
+    for (int i = tid; i < d; i += kPrecheckThreads) acc = fmaf(__ldg(w + i), load_act<T>(hg, i), acc);
+  }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
   if (lane == 0) part[warp] = acc;
@@ -80,12 +117,14 @@ extern "C" int rgd_residual_precheck(int32_t groups, int32_t d, int32_t dtype, c
   if (groups == 0) return RGD_OK;
   RGD_CHECK_ARG(h != nullptr && w != nullptr && state != nullptr, "rgd_residual_precheck: h/w/state NULL");
   cudaStream_t st = (cudaStream_t)stream;
-  if (dtype == RGD_F32)
-    precheck_kernel<float><<<groups, kPrecheckThreads, 0, st>>>(d, static_cast<const float*>(h), w, bias, theta,
-                                                                 rows_per_group, prob_out, state, row_active);
-  else
-    precheck_kernel<uint16_t><<<groups, kPrecheckThreads, 0, st>>>(d, static_cast<const uint16_t*>(h), w, bias,
-                                                                    theta, rows_per_group, prob_out, state, row_active);
-  cudaError_t e = cudaGetLastError();
+  // rows of whole 16-byte vectors, where each starts on 16 bytes
+  const bool vec = d % (dtype == RGD_F32 ? 4 : 8) == 0 && aligned16(h) && aligned16(w);
+  const cudaError_t e =
+      dtype == RGD_F32
+          ? launch_dependent(precheck_kernel<float>, groups, kPrecheckThreads, 0, st, d, vec, static_cast<const float*>(h),
+                             w, bias, theta, rows_per_group, prob_out, state, row_active)
+          : launch_dependent(precheck_kernel<uint16_t>, groups, kPrecheckThreads, 0, st, d, vec,
+                             static_cast<const uint16_t*>(h), w, bias, theta, rows_per_group, prob_out, state,
+                             row_active);
   return e == cudaSuccess ? RGD_OK : cuda_error(e, "residual_precheck launch");
 }

@@ -1142,7 +1142,7 @@ int launch_gated_head(const char* fn, int32_t rows, int32_t vocab, int32_t dtype
   hp.token_out = token_out;
   hp.kept_count = kept_count;
   hp.dev_status = dev_status;
-  hp.trie = TrieView{trie->child_begin, trie->child_tok, trie->child_node, trie->confirm};
+  hp.trie = TrieView{trie->child_begin, trie->edges};
   hp.gstate = state;
   hp.gate_row_active = row_active;
   hp.rpg = rows_per_group;

@@ -17,10 +17,11 @@
 struct rgd_trie {
   int32_t num_nodes = 0;
   int32_t num_edges = 0;
-  int32_t* child_begin = nullptr;  // [num_nodes + 1]
-  int32_t* child_tok = nullptr;    // [num_edges], sorted within a node
-  int32_t* child_node = nullptr;   // [num_edges]
-  uint8_t* confirm = nullptr;      // [num_nodes]: ends a prefix of length >= min_confirm
+  int32_t* child_begin = nullptr;  // [num_nodes + 1]: first edge of a node
+  // [num_edges], sorted by token within a node: {token, node it leads to, that
+  // node's first edge, its number of edges | confirm << 31}.  One load tells all
+  // a walk needs of the next node (confirm: it ends a prefix of length >= min_confirm).
+  int4* edges = nullptr;
   int32_t max_children = 0;        // the largest number of children of a node
   int device = 0;
 };
@@ -30,21 +31,19 @@ namespace {
 
 struct TrieView {
   const int32_t* child_begin;
-  const int32_t* child_tok;
-  const int32_t* child_node;
-  const uint8_t* confirm;
+  const int4* edges;
 };
 
-// Index of `tok` among the children of `node`, or -1.
+// Index of the edge labelled `tok` out of `node`, or -1.
 __device__ __forceinline__ int32_t find_child(const TrieView& t, int32_t node, int32_t tok) {
   int32_t lo = __ldg(t.child_begin + node), hi = __ldg(t.child_begin + node + 1);
   while (lo < hi) {
     const int32_t mid = (lo + hi) >> 1;
-    const int32_t v = __ldg(t.child_tok + mid);
+    const int32_t v = __ldg(&t.edges[mid].x);
     if (v < tok) lo = mid + 1;
     else hi = mid;
   }
-  if (lo < __ldg(t.child_begin + node + 1) && __ldg(t.child_tok + lo) == tok) return lo;
+  if (lo < __ldg(t.child_begin + node + 1) && __ldg(&t.edges[lo].x) == tok) return lo;
   return -1;
 }
 
@@ -100,8 +99,8 @@ __device__ __forceinline__ void consume_token(const TrieView& t, rgd_gate_state&
   consume_token_with(s, y, eos, max_len, root_has_children, [&](int32_t tok) {
     const int32_t e = find_child(t, s.node, tok);
     if (e < 0) return make_int2(-1, 0);
-    const int32_t nd = __ldg(t.child_node + e);
-    return make_int2(nd, (int)__ldg(t.confirm + nd));
+    const int4 x = __ldg(t.edges + e);
+    return make_int2(x.y, x.w < 0 ? 1 : 0);
   });
 }
 
