@@ -111,11 +111,18 @@ class _HostTensor:
 
 
 def _call(fn, *args):
-    """Call a C entry point unless an argument is a host tensor."""
-    for a in args:
-        if isinstance(a, _HostTensor):
-            raise ValueError(f"{a.name} must be a CUDA tensor")
-    return fn(*args)
+    """Call a C entry point unless an argument is a host tensor (which ctypes
+    refuses to convert: the arguments are looked through only then)."""
+    try:
+        return fn(*args)
+    except ctypes.ArgumentError:
+        for a in args:
+            if isinstance(a, _HostTensor):
+                raise ValueError(f"{a.name} must be a CUDA tensor") from None
+        raise
+
+
+_Tensor = None  # torch.Tensor, once an argument has been checked (importing this module does not import torch)
 
 
 def _ptr(t, name: str, dtype=None, optional: bool = False, numel: Optional[int] = None):
@@ -124,6 +131,13 @@ def _ptr(t, name: str, dtype=None, optional: bool = False, numel: Optional[int] 
     touch: a smaller tensor is refused here, since the C side sees only the
     pointer.  A host tensor gives a :class:`_HostTensor`, refused by
     :func:`_call`, so that every argument's type and size is checked first."""
+    global _Tensor
+    # A call has up to 22 tensors and its launch takes about as long as checking
+    # them: one that passes every check returns here (0.45 us; 0.84 us with the
+    # checks below for each), any other goes on to the check that it fails.
+    if type(t) is _Tensor and (dtype is None or t.dtype is dtype) and t.is_contiguous() and t.is_cuda and (
+            numel is None or t.numel() >= numel):
+        return t.data_ptr()
     if t is None:
         if optional:
             return None
@@ -131,6 +145,7 @@ def _ptr(t, name: str, dtype=None, optional: bool = False, numel: Optional[int] 
     if isinstance(t, int):
         return t
     import torch
+    _Tensor = torch.Tensor
     if not isinstance(t, torch.Tensor):
         raise TypeError(f"{name}: expected a torch tensor or an int pointer")
     if dtype is not None and t.dtype not in (dtype if isinstance(dtype, tuple) else (dtype,)):
@@ -148,6 +163,9 @@ def _stream(stream) -> Optional[int]:
     if stream is None:
         import torch
         try:
+            raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)  # (without a Stream object: 2 us less)
+            if raw is not None:
+                return raw(torch.cuda.current_device())
             return torch.cuda.current_stream().cuda_stream
         except (RuntimeError, AssertionError):  # no CUDA device: the call is refused or fails in CUDA
             return None
