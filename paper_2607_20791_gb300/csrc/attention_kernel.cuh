@@ -48,14 +48,16 @@
 // copies), P in tensor memory and one ring for K and V together (us):
 //   256 groups x 2 rows, 32/8 heads, D 128, prompts of 128-8192    440 -> 359 (0.96 of the copy rate)
 //   16 x 5, 32/8, 128, 512-2048                                     36 -> 31
-//   1 x 5, 32/8, 128, 3000                                          25 -> 17.5
+//   1 x 5, 32/8, 128, 3000                                          25 -> 16
 //   12 x 9, 32/8, 128, 500-6000                                     70 -> 50
 //   4 x 9, 64/8, 128, 32768                                        202 -> 121
 //   32 x 16, 64/8, 128, 200-800                                    107 -> 90
-//   200 x 16, 4/1, 64, 50-100                                       35 -> 34
+//   200 x 16, 4/1, 64, 50-100                                       35 -> 33
 // Every wait on an mbarrier is bounded; a timeout is reported in the status
 // word and every role stops.
 #pragma once
+
+#include <type_traits>
 
 #include "attention.h"
 #include "ptx.cuh"
@@ -336,130 +338,81 @@ __device__ __forceinline__ void split_bf16x2(float p0, float p1, uint32_t& hi, u
   lo = (l0 >> 16) | (l1 & 0xffff0000u);
 }
 
-// The merge of a split job by every thread of the block that holds its first
-// page, once all pieces are done: `pieces` partials, the block's own first, in
-// consecutive workspace slots (ml: stride mls, o: stride nq * D).  It sits at the
-// end of the block and an L2 round trip takes 1-2 us while other blocks stream,
-// so round trips are what counts: all (m, l) pairs come in one, by all threads,
-// into the table wt ([pieces][qb], for the qb queries that it has room for), and
-// an item -- four output columns of one query -- has eight pieces in flight, the
-// first ones already behind the table.  (One prompt split over 20 blocks: 13 us
-// with a thread per query walking the pieces, 4 us so.)
+// The merge of a split job by every warp of the block that holds its first page,
+// once all pieces are done: a warp takes a query, a lane D / 32 of its columns.
+// The block's own piece (0) has its O in shared memory, the others in consecutive
+// workspace slots (ml, which starts at the own piece: stride mls; o: stride nq * D).
+// It sits at the end of the block and an L2 round trip takes 1-2 us while other
+// blocks stream, so round trips are what counts: a lane brings a piece's (m, l),
+// the weights go round by shuffles, and the first eight pieces' columns are in
+// flight meanwhile.  (One prompt over 19 blocks, 20 queries: 4.6 us from the last
+// partial with a table of weights in shared memory and a barrier on both sides of it,
+// 2.4 so.)  A job of more than 32 pieces goes on in the same way, 32 at a time.
 template <int D>
-__device__ __noinline__ void merge_block(float2* wt, int qb, float* winv, const int32_t* wrow, const float2* ml,
-                                         const float* o, __nv_bfloat16* out, float* lse, int nq, int pieces, int tid,
-                                         int nthreads) {
-  const int mls = ml_stride(nq);
+__device__ __noinline__ void merge_job(const float* own, const int32_t* erow, const float2* ml, const float* o,
+                                       __nv_bfloat16* out, float* lse, int nq, int pieces, int warp, int nwarps) {
+  constexpr int kV = D / 32;
+  using Cols = typename std::conditional<D == 128, float4, float2>::type;
+  const int lane = threadIdx.x & 31, mls = ml_stride(nq);
 #pragma unroll 1
-  for (int q0 = 0; q0 < nq; q0 += qb) {
-    const int n = min(qb, nq - q0);
-    const int items = n * (D / 4);
-    const float4* src = reinterpret_cast<const float4*>(o + (int64_t)q0 * D);
-    const int64_t step = (int64_t)nq * (D / 4);
-    // a round is eight loads: pieces k0 .. k0 + 3 of two items when there are at
-    // most four, else pieces k0 .. k0 + 7 of one
-    const bool two = pieces <= 4;
-    float4 v[8];
-    auto load = [&](int i, int k0) {
+  for (int q = warp; q < nq; q += nwarps) {
+    const Cols* src = reinterpret_cast<const Cols*>(o + (int64_t)q * D) + lane;
+    const int64_t step = (int64_t)nq * 32;
+    float M = -INFINITY, l = 0.f, acc[kV];
+    {
+      const Cols x = reinterpret_cast<const Cols*>(own + q * D)[lane];
 #pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        const int k = two ? u & 3 : k0 + u, x = two && u >= 4 ? i + nthreads : i;
-        if (k < pieces && x < items) v[u] = __ldcg(src + k * step + x);
-      }
-    };
-    if (tid < items) load(tid, 0);  // (behind the table)
-#pragma unroll 2
-    for (int i = tid; i < pieces * n; i += nthreads) {
-      const int k = i / n, q = i - k * n;
-      wt[k * qb + q] = __ldcg(ml + (int64_t)k * mls + q0 + q);
+      for (int i = 0; i < kV; ++i) acc[i] = reinterpret_cast<const float*>(&x)[i];
     }
-    __syncthreads();
-    // one query per warp: its maximum, the pieces' weights (in place of m) and the sum
 #pragma unroll 1
-    for (int q = tid >> 5; q < n; q += nthreads >> 5) {
-      const int lane = tid & 31;
-      float M = -INFINITY, l = 0.f;
-#pragma unroll 1
-      for (int k = lane; k < pieces; k += 32)
-        if (wt[k * qb + q].y > 0.f) M = fmaxf(M, wt[k * qb + q].x);
+    for (int k0 = 0; k0 < pieces; k0 += 32) {
+      const int n = min(32, pieces - k0);
+      Cols v[8];
+      auto load = [&](int b) {
 #pragma unroll
-      for (int o2 = 16; o2 > 0; o2 >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, o2));
+        for (int u = 0; u < 8; ++u)
+          if (k0 + b + u > 0 && b + u < n) v[u] = __ldcg(src + (k0 + b + u) * step);
+      };
+      float2 x = make_float2(0.f, 0.f);
+      if (lane < n) x = __ldcg(ml + (int64_t)(k0 + lane) * mls + q);
+      load(0);
+      float m = x.y > 0.f ? x.x : -INFINITY;
 #pragma unroll 1
-      for (int k = lane; k < pieces; k += 32) {
-        const float2 x = wt[k * qb + q];
-        const float w = x.y > 0.f ? exp2f(x.x - M) : 0.f;
-        wt[k * qb + q].x = w;
-        l += w * x.y;
-      }
+      for (int i = 16; i > 0; i >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, i));
+      m = fmaxf(m, M);
+      const float w = x.y > 0.f ? exp2f(x.x - m) : 0.f;
+      float ls = w * x.y;
+#pragma unroll 1
+      for (int i = 16; i > 0; i >>= 1) ls += __shfl_xor_sync(0xffffffffu, ls, i);
+      // what has been summed so far (the own piece at first) comes under the new maximum
+      const float f = k0 == 0 ? __shfl_sync(0xffffffffu, w, 0) : M == -INFINITY ? 0.f : exp2f(M - m);
+      l = (k0 == 0 ? 0.f : l * f) + ls;
+      M = m;
 #pragma unroll
-      for (int o2 = 16; o2 > 0; o2 >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o2);
-      if (lane == 0) {
-        winv[q0 + q] = l > 0.f ? 1.f / l : 0.f;
-        const int row = wrow[q0 + q];
-        if (lse && row >= 0) lse[row] = l > 0.f ? (M + log2f(l)) * kLn2 : -INFINITY;
-      }
-    }
-    __syncthreads();
-    auto put = [&](int i, int q, const float4& x) {
-      const int row = wrow[q0 + q];
-      if (row < 0) return;
-      const float iv = winv[q0 + q];
-      uint2 pk;
-      pk.x = pack_bf16x2(x.x * iv, x.y * iv);
-      pk.y = pack_bf16x2(x.z * iv, x.w * iv);
-      reinterpret_cast<uint2*>(out + (int64_t)row * D)[i - q * (D / 4)] = pk;
-    };
+      for (int i = 0; i < kV; ++i) acc[i] *= f;
 #pragma unroll 1
-    for (int i = tid; i < items; i += two ? 2 * nthreads : nthreads) {
-      const int q = i / (D / 4), i2 = i + nthreads, q2 = i2 / (D / 4);
-      float4 s = make_float4(0.f, 0.f, 0.f, 0.f), s2 = s;
-#pragma unroll 1
-      for (int k0 = 0; k0 < pieces; k0 += 8) {
-        if (i != tid || k0 > 0) load(i, k0);
+      for (int b = 0; b < n; b += 8) {
+        if (b > 0) load(b);
 #pragma unroll
         for (int u = 0; u < 8; ++u) {
-          const int k = two ? u & 3 : k0 + u;
-          if (k >= pieces) continue;
-          if (two && u >= 4) {
-            if (i2 >= items) continue;
-            const float w = wt[k * qb + q2].x;
-            s2.x += w * v[u].x, s2.y += w * v[u].y, s2.z += w * v[u].z, s2.w += w * v[u].w;
-          } else {
-            const float w = wt[k * qb + q].x;
-            s.x += w * v[u].x, s.y += w * v[u].y, s.z += w * v[u].z, s.w += w * v[u].w;
+          const float wk = __shfl_sync(0xffffffffu, w, b + u);
+          if (k0 + b + u > 0 && b + u < n) {
+#pragma unroll
+            for (int i = 0; i < kV; ++i) acc[i] += wk * reinterpret_cast<const float*>(&v[u])[i];
           }
         }
       }
-      put(i, q, s);
-      if (two && i2 < items) put(i2, q2, s2);
     }
-    __syncthreads();  // (the table is rewritten for the next queries)
-  }
-}
-
-// The same for a job of so many pieces (thousands of blocks asked for) that not
-// even one query's weights fit: every element from global memory.
-template <int D>
-__device__ __noinline__ void merge_many(const int32_t* wrow, const float2* ml, const float* o, __nv_bfloat16* out,
-                                        float* lse, int nq, int pieces, int tid, int nthreads) {
-  const int mls = ml_stride(nq);
-#pragma unroll 1
-  for (int i = tid; i < nq * D; i += nthreads) {
-    const int q = i / D, d = i - q * D;
-    float M = -INFINITY, l = 0.f, v = 0.f;
-#pragma unroll 1
-    for (int k = 0; k < pieces; ++k) {
-      const float2 x = __ldcg(ml + (int64_t)k * mls + q);
-      if (!(x.y > 0.f)) continue;
-      const float Mn = fmaxf(M, x.x), f = M == -INFINITY ? 0.f : exp2f(M - Mn), w = exp2f(x.x - Mn);
-      l = l * f + w * x.y;
-      v = v * f + w * __ldcg(o + (int64_t)k * nq * D + i);
-      M = Mn;
-    }
-    const int row = wrow[q];
+    const int row = erow[q];
     if (row < 0) continue;
-    out[(int64_t)row * D + d] = __float2bfloat16(l > 0.f ? v / l : 0.f);
-    if (lse && d == 0) lse[row] = l > 0.f ? (M + log2f(l)) * kLn2 : -INFINITY;
+    const float inv = l > 0.f ? 1.f / l : 0.f;
+    uint32_t pk[kV / 2];
+#pragma unroll
+    for (int i = 0; i < kV / 2; ++i) pk[i] = pack_bf16x2(acc[2 * i] * inv, acc[2 * i + 1] * inv);
+    uint32_t* dst = reinterpret_cast<uint32_t*>(out + (int64_t)row * D) + lane * (kV / 2);
+    if constexpr (kV == 4) *reinterpret_cast<uint2*>(dst) = make_uint2(pk[0], pk[1]);
+    else *dst = pk[0];
+    if (lse && lane == 0) lse[row] = l > 0.f ? (M + log2f(l)) * kLn2 : -INFINITY;
   }
 }
 
@@ -861,8 +814,8 @@ __global__ void __launch_bounds__(AttnCfg<D, NS, QS>::kThreads, 1)
     if (is_v) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     // The split job that starts in this block is merged here, with the block's
     // last piece: its other pieces are the first ones of later blocks, behind no
-    // wait on another block, so this wait ends (bounded anyway).  Their partials
-    // are copied to the K ring, which nothing uses after the last QK.
+    // wait on another block, so waiting for them ends (bounded anyway).  Their
+    // partials, if few, are copied to the K ring, which nothing uses after the last QK.
     if (!is_v && lane == 0 && b < e) {
       const Job jb = ctx.jl;
       const int nparts = cta_of(ctx, jb.start + jb.n - 1) - c;
@@ -870,9 +823,10 @@ __global__ void __launch_bounds__(AttnCfg<D, NS, QS>::kThreads, 1)
         const int j = jb.g * p.Hkv + jb.h;
         s_mpieces = nparts + 1;
         s_mjob = j;
-        if (nparts > p.fold) mbar_arrive(&m_full);  // (nothing to wait for before the own partial)
-        int tick = wait_ticket(p.ticket + j, nparts, abort_flag, p.wait_ns);
-        if (nparts <= p.fold) {
+        if (nparts > p.fold) {
+          mbar_arrive(&m_full);  // (nothing to wait for here: the merge comes after the own partial)
+        } else {
+          int tick = wait_ticket(p.ticket + j, nparts, abort_flag, p.wait_ns);
 #pragma unroll 1
           for (int g = max(0, gbase - hk); g < gbase; ++g)
             if (!wait_or_abort(&k_empty[g % hk], (uint32_t)(g / hk) & 1u, abort_flag, p.wait_ns)) tick = -1;
@@ -889,7 +843,6 @@ __global__ void __launch_bounds__(AttnCfg<D, NS, QS>::kThreads, 1)
             mbar_arrive(&m_full);
           }
         }
-        s_tick = tick;
       }
     }
   } else if (warp == C::kQk) {
@@ -1315,8 +1268,8 @@ __global__ void __launch_bounds__(AttnCfg<D, NS, QS>::kThreads, 1)
           mbar_arrive(&ml_empty[mb]);
         }
         if (et == 96 && split) {  // (a later piece follows, so this job ends here; the last warp has least to do)
-          __threadfence();  // the partial (written by every piece-end warp before the barrier), before its count
-          atomicAdd(p.ticket + j, good && !*abort_flag ? 1 : 0x10001);
+          // the partial was written by every piece-end warp before the barrier
+          red_release_gpu_add(p.ticket + j, good && !*abort_flag ? 1 : 0x10001);
         }
         cur = nx1;
         n_in = n1;
@@ -1335,28 +1288,30 @@ __global__ void __launch_bounds__(AttnCfg<D, NS, QS>::kThreads, 1)
     if (warp < C::kEpi + 4 && s_last_ok == 2 && d < D)
       write_columns<D>(tmem + ((uint32_t)((warp & 3) * 32) << 16) + C::kOCol + 2 * s_last_ob * C::kN, C::kN,
                        (warp >> 2) * 8, (NS + 1) * 8, p.nq,
-                       split && !fold ? p.slot_o + ((int64_t)c + j) * p.nq * D + d : nullptr, p.out + d, erow, einv,
+                       parts > 0 ? (fold ? nullptr : reinterpret_cast<float*>(smem) + d)
+                       : split   ? p.slot_o + ((int64_t)c + j) * p.nq * D + d
+                                 : nullptr,
+                       p.out + d, erow, einv,
                        fold ? parts : 0, reinterpret_cast<const float*>(smem + L.kring) + d, pml_of(parts));
     tc_fence_before();
     __syncthreads();
   }
   // (a split job's last piece counts itself also when this block has given up)
-  if (tid == 0 && s_last_split > 0 && parts < 0) {
-    __threadfence();  // the partial (written by every warp before the barrier), before its count
-    atomicAdd(p.ticket + (s_last_split - 1), s_last_ok == 2 && !*abort_flag ? 1 : 0x10001);
-  }
+  if (tid == 0 && s_last_split > 0 && parts < 0)  // the partial was written by every warp before the barrier
+    red_release_gpu_add(p.ticket + (s_last_split - 1), s_last_ok == 2 && !*abort_flag ? 1 : 0x10001);
   if (parts > 0) {  // (uniform) the merge of the split job that starts in this block
     const int j = s_mjob;
-    const bool good = !fold && s_tick > 0 && (s_tick >> 16) == 0 && s_last_ok == 2 && !*abort_flag;
-    const int64_t slot = (int64_t)c + j;
-    // (the rings and P^T are idle: the table goes there)
-    const int qb = min(p.nq, L.q / 8 / s_mpieces);
-    const float2* ml = p.slot_ml + slot * ml_stride(p.nq);
-    const float* po = p.slot_o + slot * p.nq * D;
-    if (good && qb > 0)
-      merge_block<D>(reinterpret_cast<float2*>(smem), qb, einv, erow, ml, po, p.out, p.lse, p.nq, s_mpieces, tid, kThr);
-    else if (good)
-      merge_many<D>(erow, ml, po, p.out, p.lse, p.nq, s_mpieces, tid, kThr);
+    if (!fold) {
+      int tick = 0;
+      if (lane == 0) tick = wait_ticket(p.ticket + j, parts, abort_flag, p.wait_ns);
+      tick = __shfl_sync(0xffffffffu, tick, 0);
+      __syncwarp();
+      const int64_t slot = (int64_t)c + j;
+      if (tick > 0 && (tick >> 16) == 0 && s_last_ok == 2)  // (the own O is in the rings, idle by now)
+        merge_job<D>(reinterpret_cast<const float*>(smem), erow, p.slot_ml + slot * ml_stride(p.nq),
+                     p.slot_o + slot * p.nq * D, p.out, p.lse, p.nq, parts + 1, warp, kThr / 32);
+      __syncthreads();  // (every warp has seen the ticket)
+    }
     if (tid == 0) p.ticket[j] = 0;  // every other piece has counted itself
   }
   if (*abort_flag) {

@@ -113,6 +113,12 @@ __device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t b
       : "memory");
 }
 
+// Adds v to a counter in global memory after everything this thread has written or
+// has seen written (barriers) is visible to the device.
+__device__ __forceinline__ void red_release_gpu_add(int32_t* p, int32_t v) {
+  asm volatile("red.release.gpu.global.add.s32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+}
+
 // Orders this thread's generic-proxy view of global memory before its later
 // async-proxy (bulk copy) reads of it.
 __device__ __forceinline__ void fence_proxy_async_global() {

@@ -1,8 +1,8 @@
 """The attention kernel at the edges of its splits: queries per kv head on both
 sides of every softmax-set configuration, reference maxima that move in the
-middle of a job, merges of many pieces, blocks with several small jobs, and the
-two forms kept for extreme calls (suffix lengths left in global memory, a job of
-more pieces than have room for their weights).  Against the fp64 oracle with the
+middle of a job, merges of many pieces, blocks with several small jobs, and
+extreme calls (suffix lengths left in global memory, a job of thousands of
+pieces).  Against the fp64 oracle with the
 bounds of the other attention tests."""
 import numpy as np
 import pytest
@@ -82,6 +82,6 @@ def test_suffix_lengths_in_global_memory(gpu_lib):
 
 
 def test_job_of_thousands_of_pieces(gpu_lib):
-    # a page per block: more pieces than the merge has room for weights
+    # a page per block: a merge of hundreds of rounds
     case = workloads.make_attn_case("pieces", 1, 2, 2, 1, 64, [330000], [5, 20], seed=12)
     _check(case, _run(case, num_ctas=40000))
