@@ -215,6 +215,10 @@ extern "C" int rgd_prefix_decode_attn(const rgd_attn_shape* shape, const rgd_bf1
   p.nq = pl.nq;
   p.C = pl.C;
   p.hk = pl.hk;
+  auto mul_of = [](int n) { return ((1ull << 32) + n - 1) / n; };
+  p.rpg_mul = mul_of(s.rows_per_group);  // (at most kSmemLimit / 8 groups of 128 rows: x n < 2^32)
+  p.hk_mul = mul_of(pl.hk);
+  p.hv_mul = mul_of(pl.hv);
   p.hv = pl.hv;
   p.np = pl.np;
   p.nqb = pl.nqb;

@@ -47,12 +47,12 @@
 // graph, against a kernel with the queries as the MMA's M (128 rows of query
 // copies), P in tensor memory and one ring for K and V together (us):
 //   256 groups x 2 rows, 32/8 heads, D 128, prompts of 128-8192    440 -> 359 (0.96 of the copy rate)
-//   16 x 5, 32/8, 128, 512-2048                                     36 -> 31
-//   1 x 5, 32/8, 128, 3000                                          25 -> 16
-//   12 x 9, 32/8, 128, 500-6000                                     70 -> 50
-//   4 x 9, 64/8, 128, 32768                                        202 -> 121
-//   32 x 16, 64/8, 128, 200-800                                    107 -> 90
-//   200 x 16, 4/1, 64, 50-100                                       35 -> 33
+//   16 x 5, 32/8, 128, 512-2048                                     36 -> 30
+//   1 x 5, 32/8, 128, 3000                                          25 -> 15.3
+//   12 x 9, 32/8, 128, 500-6000                                     70 -> 48
+//   4 x 9, 64/8, 128, 32768                                        202 -> 119
+//   32 x 16, 64/8, 128, 200-800                                    107 -> 87
+//   200 x 16, 4/1, 64, 50-100                                       35 -> 32
 // Every wait on an mbarrier is bounded; a timeout is reported in the status
 // word and every role stops.
 #pragma once
@@ -158,24 +158,26 @@ __device__ __forceinline__ int slen_of(const BlockCtx& c, int r) {
   return row_bit(c.rowbits, r) ? clamp_len(__ldg(c.suffix_len + r), c.max_sp) : 0;
 }
 
+// An active row's suffix pages into its group's count (word g + 1 of gpre, whose top
+// bit says that a row of the group is active).
+constexpr uint32_t kAnyActive = 0x80000000u;
+__device__ __forceinline__ void count_row(const AttnParams& p, int32_t* gpre, int r, int slen) {
+  const int g = (int)(((uint64_t)(uint32_t)r * p.rpg_mul) >> 32);
+  uint32_t* w = reinterpret_cast<uint32_t*>(gpre + g + 1);
+  atomicAdd(w, (uint32_t)pages_of(slen));
+  atomicOr(w, kAnyActive);
+}
 // A group's pages: its prompt pages if any row of it is active, plus its active
 // rows' suffix pages.
-__device__ __noinline__ int group_pages(const BlockCtx& c, int g) {
-  int n = 0;
-  bool any = false;
-#pragma unroll 4
-  for (int r = g * c.rpg; r < (g + 1) * c.rpg; ++r) {
-    n += pages_of(slen_of(c, r));
-    any = any || row_bit(c.rowbits, r);
-  }
-  return any ? n + pages_of(c.plen[g]) : 0;
+__device__ __forceinline__ int pages_of_group(int word, int plen) {
+  return word < 0 ? (int)((uint32_t)word & ~kAnyActive) + pages_of(plen) : 0;
 }
 
 // The lengths and activity of the rows past the first one per thread (G <= rows),
 // four of a thread's rows in flight.  Out of line: a call with few rows does not
 // fetch this code.
-__device__ __noinline__ void more_rows(const AttnParams& p, int32_t* slen_s, int32_t* plen_s, uint32_t* rowbits, int c,
-                                       int tid, int nthreads) {
+__device__ __noinline__ void more_rows(const AttnParams& p, int32_t* slen_s, int32_t* plen_s, uint32_t* rowbits,
+                                       int32_t* gpre, int c, int tid, int nthreads) {
   constexpr int kU = 4;
   const int lane = tid & 31, nrows = p.G * p.rpg;
 #pragma unroll 1
@@ -196,7 +198,9 @@ __device__ __noinline__ void more_rows(const AttnParams& p, int32_t* slen_s, int
       const int r = r0 + u * nthreads;
       if (r < nrows) {
         if (c == 0 && (sl[u] < 0 || sl[u] > p.max_sp * kPage)) flag(p.dev_status, RGD_DEV_BAD_PAGE);
-        if (p.slen_in_smem) slen_s[r] = act[u] ? clamp_len(sl[u], p.max_sp) : 0;
+        sl[u] = act[u] ? clamp_len(sl[u], p.max_sp) : 0;
+        if (p.slen_in_smem) slen_s[r] = sl[u];
+        if (act[u]) count_row(p, gpre, r, sl[u]);
         if (r < p.G) {
           if (c == 0 && (pl[u] < 0 || pl[u] > p.max_pp * kPage)) flag(p.dev_status, RGD_DEV_BAD_PAGE);
           plen_s[r] = clamp_len(pl[u], p.max_pp);
@@ -620,6 +624,9 @@ __global__ void __launch_bounds__(AttnCfg<D, NS, QS>::kThreads, 1)
     prefetch_tensormap(&tmK);
     prefetch_tensormap(&tmV);
   }
+#pragma unroll 1
+  for (int g = tid; g <= p.G; g += kThr) gpre[g] = 0;
+  __syncthreads();
   // launched as a programmatic dependent of the previous kernel on the stream:
   // everything below may read what that kernel wrote
   asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -651,7 +658,9 @@ __global__ void __launch_bounds__(AttnCfg<D, NS, QS>::kThreads, 1)
     auto store = [&](int r) {
       if (r < nrows) {
         if (c == 0 && (sl < 0 || sl > p.max_sp * kPage)) flag(p.dev_status, RGD_DEV_BAD_PAGE);
-        if (p.slen_in_smem) slen_s[r] = act ? clamp_len(sl, p.max_sp) : 0;
+        sl = act ? clamp_len(sl, p.max_sp) : 0;
+        if (p.slen_in_smem) slen_s[r] = sl;
+        if (act) count_row(p, gpre, r, sl);
       }
       if (r < p.G) {
         if (c == 0 && (pl < 0 || pl > p.max_pp * kPage)) flag(p.dev_status, RGD_DEV_BAD_PAGE);
@@ -661,10 +670,9 @@ __global__ void __launch_bounds__(AttnCfg<D, NS, QS>::kThreads, 1)
       if (lane == 0 && r - lane < nrows) rowbits[r >> 5] = bits;
     };
     store(tid);
-    if (nrows > kThr) more_rows(p, slen_s, plen_s, rowbits, c, tid, kThr);
+    if (nrows > kThr) more_rows(p, slen_s, plen_s, rowbits, gpre, c, tid, kThr);
   }
   if (tid == 0) {
-    gpre[0] = 0;
     ctx.G = p.G;
     ctx.Hkv = p.Hkv;
     ctx.rpg = p.rpg;
@@ -679,20 +687,22 @@ __global__ void __launch_bounds__(AttnCfg<D, NS, QS>::kThreads, 1)
     ctx.rowbits = rowbits;
   }
   __syncthreads();
-  if (p.G > 32) {
-#pragma unroll 1
-    for (int g = tid; g < p.G; g += kThr) gpre[g + 1] = group_pages(ctx, g);
-    __syncthreads();
-  }
-  if (warp == 0) {  // inclusive prefix sum of gpre[1..G], then this block's range
+  if (warp == 0) {  // inclusive prefix sum of the groups' pages, then this block's range
+    // (up to 32 groups, one per lane, stay in registers; every function called or
+    // division made here is on the path to the first copy, and cold)
+    const bool few = p.G <= 32;
     const int E = (p.G + 31) / 32;
     const int lo = 1 + lane * E, hi = min(p.G + 1, lo + E);
     int sum = 0;
-    if (p.G <= 32) {
-      if (lane < p.G) sum = group_pages(ctx, lane);
+    if (few) {
+      if (lane < p.G) sum = pages_of_group(gpre[lane + 1], plen_s[lane]);
     } else {
 #pragma unroll 1
-      for (int i = lo; i < hi; ++i) sum += gpre[i];
+      for (int i = lo; i < hi; ++i) {
+        const int n = pages_of_group(gpre[i], plen_s[i - 1]);
+        gpre[i] = n;
+        sum += n;
+      }
     }
     int incl = sum;
 #pragma unroll
@@ -700,7 +710,7 @@ __global__ void __launch_bounds__(AttnCfg<D, NS, QS>::kThreads, 1)
       const int v = __shfl_up_sync(0xffffffffu, incl, o);
       if (lane >= o) incl += v;
     }
-    if (p.G <= 32) {
+    if (few) {
       if (lane < p.G) gpre[lane + 1] = incl;
     } else {
       int run = incl - sum;
@@ -713,7 +723,7 @@ __global__ void __launch_bounds__(AttnCfg<D, NS, QS>::kThreads, 1)
     __syncwarp();
     // pages are divided over Ceff = min(C, T) blocks so that every working block
     // has at least one page (a job's pieces are then exactly the blocks first..last)
-    const int T = p.Hkv * gpre[p.G], Ceff = min(p.C, T);
+    const int T = p.Hkv * __shfl_sync(0xffffffffu, incl, 31), Ceff = min(p.C, T);
     int x = T;  // lane 0: b; lane 1: e
     if (c < Ceff && lane < 2) x = div_nn((int64_t)(c + lane) * T, Ceff);
     const int b = __shfl_sync(0xffffffffu, x, 0), e = __shfl_sync(0xffffffffu, x, 1);
@@ -725,7 +735,19 @@ __global__ void __launch_bounds__(AttnCfg<D, NS, QS>::kThreads, 1)
     }
     __syncwarp();
     if (b < e) {  // the jobs at the range's ends (lanes 0 and 1)
-      const Job j = job_at(ctx, lane == 1 ? e - 1 : b);
+      const int at = lane == 1 ? e - 1 : b;
+      Job j;
+      if (few) {  // (lane g holds the prefix sum up to group g)
+        const int g0 = __popc(__ballot_sync(0xffffffffu, lane < p.G && p.Hkv * incl <= b));
+        const int g1 = __popc(__ballot_sync(0xffffffffu, lane < p.G && p.Hkv * incl < e));
+        j.g = lane == 1 ? g1 : g0;
+        j.n = __shfl_sync(0xffffffffu, sum, j.g);
+        const int base = p.Hkv * (__shfl_sync(0xffffffffu, incl, j.g) - j.n);
+        j.h = (int)((uint32_t)(at - base) / (uint32_t)j.n);
+        j.start = base + j.h * j.n;
+      } else {
+        j = job_at(ctx, at);
+      }
       if (lane == 0) {
         ctx.j0 = j;
         ctx.n0 = min(e, j.start + j.n) - b;
@@ -750,6 +772,7 @@ __global__ void __launch_bounds__(AttnCfg<D, NS, QS>::kThreads, 1)
     // first wait of a round, so the block-table loads are in flight meanwhile.
     const bool is_v = warp == C::kProdV;
     const int nr = is_v ? hv : hk;
+    const uint64_t nr_mul = is_v ? p.hv_mul : p.hk_mul;
     uint64_t* full = is_v ? v_full : k_full;
     uint64_t* empty = is_v ? v_empty : k_empty;
     uint8_t* ring = smem + (is_v ? L.vring : L.kring);
@@ -770,7 +793,7 @@ __global__ void __launch_bounds__(AttnCfg<D, NS, QS>::kThreads, 1)
         const int g0 = __shfl_sync(0xffffffffu, gidx, 0);
         const int g1 = __shfl_sync(0xffffffffu, gidx, 31 - __clz(__ballot_sync(0xffffffffu, valid)));
         gbase += __popc(starts);
-        const int gs = gidx % nr;
+        const int gs = gidx - (int)(((uint64_t)(uint32_t)gidx * nr_mul) >> 32) * nr;  // gidx % nr
         bool aborted = false;
 #pragma unroll 1
         for (int gq = g0; gq <= g1; ++gq) {
