@@ -214,6 +214,15 @@ extern "C" int rgd_prefix_decode_attn(const rgd_attn_shape* shape, const rgd_bf1
   p.max_sp = s.max_suffix_pages;
   p.nq = pl.nq;
   p.C = pl.C;
+  // A job's end takes its block's warps about 2300 cycles and more with many
+  // queries, a page 340 cycles at head dim 128 and the copy rate.  In pages, 0 / 6 /
+  // 16: 16 groups x 5 rows 30.4 / 29.7 / 30.2 us; 32 x 16 rows of 128 queries a job
+  // 87.6 / 83.9 / 82.8; 32 x 4 rows at head dim 64 37.3 / 36.5 / 35.4.
+  p.end_pages = (6 + pl.nq / 16) * 128 / s.head_dim;
+  if (((int64_t)s.num_groups * (s.max_prompt_pages + (int64_t)s.rows_per_group * s.max_suffix_pages + p.end_pages)) *
+          s.num_kv_heads >=
+      (int64_t)1 << 31)
+    p.end_pages = 0;  // (the positions must fit 31 bits)
   p.hk = pl.hk;
   auto mul_of = [](int n) { return ((1ull << 32) + n - 1) / n; };
   p.rpg_mul = mul_of(s.rows_per_group);  // (at most kSmemLimit / 8 groups of 128 rows: x n < 2^32)

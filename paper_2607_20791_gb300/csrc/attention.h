@@ -97,6 +97,7 @@ struct AttnParams {
   int32_t* dev_status;
   int32_t G, rpg, Hq, Hkv, gq, num_pages, max_pp, max_sp;
   int32_t nq, C;
+  int32_t end_pages;     // pages that a job's end counts for when the pages are dealt to the blocks
   int32_t hk, hv;        // K and V areas of the ring
   uint64_t rpg_mul, hk_mul, hv_mul;  // ceil(2^32 / rpg), / hk, / hv: x / n = x n_mul >> 32 while x n < 2^32
   int32_t np, nqb;       // P^T and Q buffers (1 or 2)

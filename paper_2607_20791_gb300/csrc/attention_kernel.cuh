@@ -46,12 +46,12 @@
 // -> block table -> data) and the merge at the end.  Measured inside a CUDA
 // graph, against a kernel with the queries as the MMA's M (128 rows of query
 // copies), P in tensor memory and one ring for K and V together (us):
-//   256 groups x 2 rows, 32/8 heads, D 128, prompts of 128-8192    440 -> 359 (0.96 of the copy rate)
-//   16 x 5, 32/8, 128, 512-2048                                     36 -> 30
+//   256 groups x 2 rows, 32/8 heads, D 128, prompts of 128-8192    440 -> 355 (0.97 of the copy rate)
+//   16 x 5, 32/8, 128, 512-2048                                     36 -> 29.5
 //   1 x 5, 32/8, 128, 3000                                          25 -> 15.3
-//   12 x 9, 32/8, 128, 500-6000                                     70 -> 48
-//   4 x 9, 64/8, 128, 32768                                        202 -> 119
-//   32 x 16, 64/8, 128, 200-800                                    107 -> 87
+//   12 x 9, 32/8, 128, 500-6000                                     70 -> 47
+//   4 x 9, 64/8, 128, 32768                                        202 -> 118
+//   32 x 16, 64/8, 128, 200-800                                    107 -> 83
 //   200 x 16, 4/1, 64, 50-100                                       35 -> 32
 // Every wait on an mbarrier is bounded; a timeout is reported in the status
 // word and every role stops.
@@ -98,7 +98,9 @@ struct Job {
 // take it are out of line and shared by the roles, which keeps the kernel's code
 // (fetched cold by every launch) small.
 struct BlockCtx {
-  int b, e, T, Ceff;  // this block's pages [b, e) of T, which Ceff blocks share
+  int b, e;        // this block's pages
+  int T, Ceff;     // the dealt pages (see the set-up), which Ceff blocks share
+  int jl_end;      // dealt position of the last job's last page
   int G, Hkv, rpg, max_pp, max_sp;
   const int32_t *prompt_bt, *suffix_bt, *suffix_len;
   const int32_t *gpre, *plen, *slen;  // slen: NULL when it is read from global memory
@@ -139,9 +141,6 @@ __device__ __noinline__ Job job_at(const BlockCtx& c, int x) {
   j.start = base + j.h * j.n;
   return j;
 }
-
-// Block whose page range contains global page x (ranges [floor(cT/C), floor((c+1)T/C))).
-__device__ __noinline__ int cta_of(const BlockCtx& c, int x) { return div_nn((int64_t)(x + 1) * c.Ceff - 1, c.T); }
 
 // The piece after (cur, n pages): its job and pages; false when there is none.
 __device__ __noinline__ bool next_piece(const BlockCtx& c, Job& cur, int& n) {
@@ -721,11 +720,36 @@ __global__ void __launch_bounds__(AttnCfg<D, NS, QS>::kThreads, 1)
       }
     }
     __syncwarp();
-    // pages are divided over Ceff = min(C, T) blocks so that every working block
-    // has at least one page (a job's pieces are then exactly the blocks first..last)
-    const int T = p.Hkv * __shfl_sync(0xffffffffu, incl, 31), Ceff = min(p.C, T);
-    int x = T;  // lane 0: b; lane 1: e
-    if (c < Ceff && lane < 2) x = div_nn((int64_t)(c + lane) * T, Ceff);
+    // The pages are dealt over Ceff = min(C, T) blocks, block c taking the positions
+    // [floor(c T / Ceff), floor((c + 1) T / Ceff)) of T.  With up to 32 groups (more
+    // give every block about as many job ends) and more pages than blocks, every job
+    // counts p.end_pages more than it has, for the time of its end, so that a block
+    // with more ends gets fewer pages; positions past a job's pages map to its end.  Every position is some block's, so a job's pieces are exactly the blocks
+    // from that of its first page to that of its last.
+    const int pages = p.Hkv * __shfl_sync(0xffffffffu, incl, 31);
+    const int extra = few && pages > p.C ? p.end_pages : 0;
+    const uint32_t some = __ballot_sync(0xffffffffu, few && sum > 0);
+    const int ends = __popc(some & (0xffffffffu >> (31 - lane)));  // groups with pages, up to the lane's
+    const int vincl = p.Hkv * (incl + extra * ends);
+    const int T = __shfl_sync(0xffffffffu, vincl, 31), Ceff = min(p.C, T);
+    int x = pages;  // lane 0: b; lane 1: e
+    auto group_of = [&](int v, int at0, int at1) {  // the group in which lane 0's (1's) position lies, by prefix sums v
+      const int g0 = __popc(__ballot_sync(0xffffffffu, lane < p.G && v <= at0));
+      const int g1 = __popc(__ballot_sync(0xffffffffu, lane < p.G && v <= at1));
+      return lane == 1 ? g1 : g0;
+    };
+    if (c < Ceff) {
+      const int y = div_nn((int64_t)(c + (lane & 1)) * T, Ceff);
+      if (extra == 0) {
+        x = y;
+      } else {
+        const int g = group_of(vincl, __shfl_sync(0xffffffffu, y, 0), __shfl_sync(0xffffffffu, y, 1));
+        const int n = __shfl_sync(0xffffffffu, sum, g), excl = __shfl_sync(0xffffffffu, incl, g) - n;
+        const int off = y - (__shfl_sync(0xffffffffu, vincl, g) - p.Hkv * (n + extra));
+        const int h = (int)((uint32_t)off / (uint32_t)max(1, n + extra));
+        if (g < p.G) x = p.Hkv * excl + h * n + min(off - h * (n + extra), n);
+      }
+    }
     const int b = __shfl_sync(0xffffffffu, x, 0), e = __shfl_sync(0xffffffffu, x, 1);
     if (lane == 0) {
       ctx.b = b;
@@ -737,22 +761,26 @@ __global__ void __launch_bounds__(AttnCfg<D, NS, QS>::kThreads, 1)
     if (b < e) {  // the jobs at the range's ends (lanes 0 and 1)
       const int at = lane == 1 ? e - 1 : b;
       Job j;
-      if (few) {  // (lane g holds the prefix sum up to group g)
-        const int g0 = __popc(__ballot_sync(0xffffffffu, lane < p.G && p.Hkv * incl <= b));
-        const int g1 = __popc(__ballot_sync(0xffffffffu, lane < p.G && p.Hkv * incl < e));
-        j.g = lane == 1 ? g1 : g0;
+      int end;
+      if (few) {  // (lane g holds the prefix sums up to group g)
+        j.g = group_of(p.Hkv * incl, b, e - 1);
         j.n = __shfl_sync(0xffffffffu, sum, j.g);
         const int base = p.Hkv * (__shfl_sync(0xffffffffu, incl, j.g) - j.n);
         j.h = (int)((uint32_t)(at - base) / (uint32_t)j.n);
         j.start = base + j.h * j.n;
+        end = __shfl_sync(0xffffffffu, vincl, j.g) - (p.Hkv - 1 - j.h) * (j.n + extra) - extra - 1;
       } else {
         j = job_at(ctx, at);
+        end = j.start + j.n - 1;
       }
       if (lane == 0) {
         ctx.j0 = j;
         ctx.n0 = min(e, j.start + j.n) - b;
       }
-      if (lane == 1) ctx.jl = j;
+      if (lane == 1) {
+        ctx.jl = j;
+        ctx.jl_end = end;
+      }
     }
   }
   tc_fence_before();
@@ -841,7 +869,7 @@ __global__ void __launch_bounds__(AttnCfg<D, NS, QS>::kThreads, 1)
     // partials, if few, are copied to the K ring, which nothing uses after the last QK.
     if (!is_v && lane == 0 && b < e) {
       const Job jb = ctx.jl;
-      const int nparts = cta_of(ctx, jb.start + jb.n - 1) - c;
+      const int nparts = div_nn((int64_t)(ctx.jl_end + 1) * ctx.Ceff - 1, ctx.T) - c;
       if (jb.start >= b && nparts > 0) {
         const int j = jb.g * p.Hkv + jb.h;
         s_mpieces = nparts + 1;

@@ -63,6 +63,23 @@ def test_fold_of_few_pieces(gpu_lib, D, rpg, heads, pieces):
     _check(case, _run(case, num_ctas=pieces + 2))
 
 
+@pytest.mark.parametrize("G", [1, 2, 31, 32, 33])
+@pytest.mark.parametrize("ctas", [2, 7, 40, 0])
+def test_pages_dealt_to_blocks(gpu_lib, G, ctas):
+    # both sides of the 32 groups up to which a job's end counts as pages, with
+    # empty and inactive groups, jobs of a page, and ends on both sides of a block's
+    # bounds (2 to about 150 blocks)
+    rng = np.random.default_rng(G * 100 + ctas)
+    plen = rng.integers(1, 400, G)
+    plen[G // 3::5] = 0
+    plen[G // 2] = 16
+    act = (rng.random(2 * G) > 0.15).astype(np.uint8)
+    act[2 * (G // 4):2 * (G // 4) + 2] = G < 2
+    case = workloads.make_attn_case("dealt", G, 2, 6, 3, 64 if G % 2 else 128, plen, rng.integers(0, 40, 2 * G),
+                                    seed=G + ctas, row_active=act)
+    _check(case, _run(case, num_ctas=ctas))
+
+
 def test_blocks_with_several_small_jobs(gpu_lib):
     # three blocks for 40 jobs of 1-4 pages: pieces follow one another with one group each
     rng = np.random.default_rng(3)
