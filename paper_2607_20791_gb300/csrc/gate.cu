@@ -11,6 +11,7 @@
 #include <cooperative_groups.h>
 
 #include <algorithm>
+#include <atomic>
 #include <climits>
 #include <cmath>
 #include <map>
@@ -153,9 +154,9 @@ __global__ void __launch_bounds__(kGateThreads)
 // the stop token, which d(q) drops -- are found, and if their probability
 // mass m reaches rho the most probable of them is appended instead.
 //
-// One thread-block cluster of kSoftCluster CTAs per group, each CTA taking an
-// equal contiguous share of the probe's logits, copied into shared memory in
-// chunks by bulk copies issued before anything else.  While they are in
+// One thread-block cluster of K CTAs per group (K by the number of groups, see
+// rgd_soft_gate), each CTA taking an equal contiguous share of the probe's logits,
+// copied into shared memory in chunks by bulk copies issued before anything else.  While they are in
 // flight, the children of the probe's trie node (token, node, confirm flag)
 // are read into shared memory -- every trie lookup of the step is then a
 // shared-memory scan -- and, when the soft branch can be taken at this step,
@@ -165,16 +166,19 @@ __global__ void __launch_bounds__(kGateThreads)
 // order.  The pass finds the maximum, its lowest index (y) and the softmax
 // normaliser Z and counts the logits above each of the kProbe best
 // candidates, which settles the prefix unless all of them are in the top K;
-// then the candidates are sorted (bitonic, in shared memory) and a binary
-// search over the rest, one more pass over the logits (from L2) per probed
-// candidate, finishes it.  After each pass every CTA pushes its partial
+// then the candidates are sorted (bitonic, in shared memory) and a search over
+// the rest finishes it, one candidate a pass: the next, then ever wider steps
+// until one is out (few are in the top K where most of a node's children are
+// improbable: one pass then, a binary search takes six for 36), then halving.  A
+// pass reads the share in shared memory if its chunks still hold all of it, else
+// from L2.  After each pass every CTA pushes its partial
 // results into every CTA's shared memory and all of them combine the same
 // values in the same order, so every CTA takes the same decisions; CTA 0
 // writes the step's outcome.  The kernel runs once per decode step behind
 // kernels that sweep L2, so its own instructions are fetched cold: its loops
 // stay rolled, which keeps the code it runs short.
 constexpr int kSoftThreads = 512;
-constexpr int kSoftCluster = 6;
+constexpr int kSoftCluster = 6;  // CTAs per group at most (6, 4 or 2)
 constexpr int kMaxCand = 2048;  // a node's children + the stop token (a power of two: the sort's padding)
 constexpr int kProbe = 4;       // candidates whose ranks the first pass counts
 constexpr int kSoftChunk = 32768;  // bytes of logits per bulk copy
@@ -343,7 +347,7 @@ __device__ __noinline__ SoftPart merge_lanes(SoftPart p, const SoftPart* parts, 
 }
 
 template <typename LT>
-__global__ void __cluster_dims__(kSoftCluster, 1, 1) __launch_bounds__(kSoftThreads, 1)
+__global__ void __launch_bounds__(kSoftThreads, 1)
     soft_gate_kernel(TrieView t, int32_t rows_per_group, int32_t vocab, const LT* __restrict__ logits,
                      int64_t row_stride, bool vec, int32_t top_k, float rho, int32_t c, int32_t eos, int32_t max_len,
                      rgd_gate_state* __restrict__ state, uint8_t* __restrict__ row_active, int32_t* token_out,
@@ -354,15 +358,15 @@ __global__ void __cluster_dims__(kSoftCluster, 1, 1) __launch_bounds__(kSoftThre
   __shared__ SoftShared sh;
   extern __shared__ uint4 soft_buf[];  // kSoftStages chunks
   cg::cluster_group cluster = cg::this_cluster();
-  const int rank = (int)cluster.block_rank();
-  const int g = blockIdx.x / kSoftCluster, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int rank = (int)cluster.block_rank(), K = (int)cluster.num_blocks();
+  const int g = blockIdx.x / K, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const LT* row = logits + (int64_t)g * row_stride;
   // this CTA's share of the row: vectors [lo, lo + nv) when the row is
   // 16-byte aligned (staged through shared memory), else elements [lo, hi_u)
   const int32_t nvec = vocab / E;
   const int32_t n_units = vec ? nvec : vocab;
-  const int32_t lo = (int32_t)((int64_t)n_units * rank / kSoftCluster);
-  const int32_t hi_u = (int32_t)((int64_t)n_units * (rank + 1) / kSoftCluster);
+  const int32_t lo = (int32_t)((int64_t)n_units * rank / K);
+  const int32_t hi_u = (int32_t)((int64_t)n_units * (rank + 1) / K);
   const int32_t nv = vec ? hi_u - lo : 0;
   const int32_t nchunks = (nv + kVpc - 1) / kVpc;
   const uint4* rv = reinterpret_cast<const uint4*>(row);
@@ -384,9 +388,12 @@ __global__ void __cluster_dims__(kSoftCluster, 1, 1) __launch_bounds__(kSoftThre
   if (tid == 0) {
     for (int b = 0; b < kSoftStages; ++b) mbar_init(&sh.full[b], 1);
     fence_mbar_init();
-    for (int32_t ck = 0; ck < min(kSoftStages, nchunks); ++ck) issue(ck);
     sh.ncand = 0;
   }
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");  // (a dependent waits for this kernel's end)
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  if (tid == 0)
+    for (int32_t ck = 0; ck < min(kSoftStages, nchunks); ++ck) issue(ck);
   // Every thread reads the state and takes the same decisions from it: the
   // kernel has no section where one warp works while the others wait.
   const rgd_gate_state s0 = state[g];
@@ -511,6 +518,7 @@ __global__ void __cluster_dims__(kSoftCluster, 1, 1) __launch_bounds__(kSoftThre
       // z, and the probes for the few logits at or above the weakest one
       if (m != -INFINITY) {
         const float ml = m * kLog2e;
+        float zc = 0.f;  // (a chunk's share: short sums round less)
 #pragma unroll 1
         for (int32_t k = tid; k < cnt; k += kSoftThreads) {
           const uint4 x = buf[k];
@@ -523,8 +531,9 @@ __global__ void __cluster_dims__(kSoftCluster, 1, 1) __launch_bounds__(kSoftThre
             if (v0 >= p_min) probe_counts(v0, (base + k) * E + e);
             if (v1 >= p_min) probe_counts(v1, (base + k) * E + e + 1);
           }
-          z += z0 + z1;
+          zc += z0 + z1;
         }
+        z += zc;
       } else if (bm >= p_min) {  // (every logit so far is -inf, and so is a probed candidate)
 #pragma unroll 1
         for (int32_t k = tid; k < cnt; k += kSoftThreads) {
@@ -540,9 +549,9 @@ __global__ void __cluster_dims__(kSoftCluster, 1, 1) __launch_bounds__(kSoftThre
     }
     // the few logits past the last whole vector
     const int32_t i = nvec * E + tid;
-    if (rank == kSoftCluster - 1 && i < vocab) one(logit_at<LT>(row, i), i);
+    if (rank == K - 1 && i < vocab) one(logit_at<LT>(row, i), i);
   } else {
-    scan_row<kSoftThreads, 8, LT>(row, vocab, false, rank, kSoftCluster, one, [] {});
+    scan_row<kSoftThreads, 8, LT>(row, vocab, false, rank, K, one, [] {});
   }
   if (timed_out && dev_status) atomicOr(dev_status, RGD_DEV_WAIT_TIMEOUT);  // (the outputs are then not valid)
 
@@ -556,7 +565,7 @@ __global__ void __cluster_dims__(kSoftCluster, 1, 1) __launch_bounds__(kSoftThre
     for (int q = 0; q < kProbe; ++q) p.c[q] = pc[q];
     p = merge_lanes(p, nullptr, 0);
     cluster_wait();  // every CTA of the cluster has started
-    if (lane < kSoftCluster) cluster.map_shared_rank(&sh, lane)->part[rank * kWarps + warp] = p;
+    if (lane < K) cluster.map_shared_rank(&sh, lane)->part[rank * kWarps + warp] = p;
   }
   cluster.sync();  // every warp's share is in every CTA's shared memory
   // ---- the same combination, in the same order, in every warp of the cluster ----
@@ -566,7 +575,7 @@ __global__ void __cluster_dims__(kSoftCluster, 1, 1) __launch_bounds__(kSoftThre
   all.mi = 0x7fffffff;
 #pragma unroll
   for (int q = 0; q < kProbe; ++q) all.c[q] = 0;
-  all = merge_lanes(all, sh.part, kSoftCluster * kWarps);
+  all = merge_lanes(all, sh.part, K * kWarps);  // (K is even: a multiple of 32)
   const int32_t y = all.mi;
   // the children labelled y and a* (the best candidate), if any
   const int32_t a_star = np_ > 0 ? pi[0] : -1;
@@ -588,9 +597,8 @@ __global__ void __cluster_dims__(kSoftCluster, 1, 1) __launch_bounds__(kSoftThre
     while (n_in < np_ && all.c[n_in] < top_k) ++n_in;
   if (soft && n_in == np_ && np_ < hi) {
     // ---- the rest: sort the candidates (bitonic, padded to a power of two;
-    // the first np_ are the probed ones), then a binary search over
-    // candidates np_ .. hi - 1, one comparison per logit per probed
-    // candidate (every thread of the cluster takes the same steps) ----
+    // the first np_ are the probed ones), then a search over
+    // candidates np_ .. hi - 1 (every thread of the cluster takes the same steps) ----
     int32_t np2 = 1;
     while (np2 < nslot) np2 <<= 1;
     for (int32_t i = nslot + tid; i < np2; i += kSoftThreads) sh.key[i] = ~0ull;
@@ -610,29 +618,47 @@ __global__ void __cluster_dims__(kSoftCluster, 1, 1) __launch_bounds__(kSoftThre
         __syncthreads();
       }
     }
-    int32_t lo_c = np_, hi_c = hi;
+    int32_t lo_c = np_, hi_c = hi, step = 1;
+    bool out = false;  // a candidate outside the top K has been found
+    const bool staged = vec && nchunks <= kSoftStages;  // (the share's chunks are contiguous and still there)
+#pragma unroll 1
     for (int pass = 0; lo_c < hi_c; ++pass) {
-      const int32_t mid = (lo_c + hi_c) >> 1;
+      const int32_t mid = out ? (lo_c + hi_c) >> 1 : min(lo_c + step - 1, hi_c - 1);
       const uint64_t key = sh.key[mid];
       const float cv = key_logit(key);
       const int32_t ci = (int32_t)(uint32_t)key;
       if (tid == 0) sh.cnt_cta = 0;
       __syncthreads();
       int32_t cnt = 0;
-      scan_row<kSoftThreads, 8, LT>(
-          row, vocab, vec, rank, kSoftCluster, [&](float v, int32_t i) { cnt += above(v, i, cv, ci) ? 1 : 0; },
-          [] {});
+      auto count = [&](float v, int32_t i) { cnt += above(v, i, cv, ci) ? 1 : 0; };
+      if (staged) {
+#pragma unroll 2
+        for (int32_t k = tid; k < nv; k += kSoftThreads) {
+          const uint4 x = soft_buf[k];
+#pragma unroll
+          for (int e = 0; e < E; ++e) count(vec_elem<LT>(x, e), (lo + k) * E + e);
+        }
+        const int32_t i = nvec * E + tid;
+        if (rank == K - 1 && i < vocab) count(logit_at<LT>(row, i), i);
+      } else {
+        scan_row<kSoftThreads, 8, LT>(row, vocab, vec, rank, K, count, [] {});
+      }
       cnt = __reduce_add_sync(0xffffffffu, cnt);
       if (lane == 0 && cnt) atomicAdd(&sh.cnt_cta, cnt);
       __syncthreads();
       // CTA r's slot of this pass's parity is next written two passes on,
       // after every CTA has passed the next cluster barrier (and read this one)
-      if (warp == 0 && lane < kSoftCluster) cluster.map_shared_rank(&sh, lane)->cnt[pass & 1][rank] = sh.cnt_cta;
+      if (warp == 0 && lane < K) cluster.map_shared_rank(&sh, lane)->cnt[pass & 1][rank] = sh.cnt_cta;
       cluster.sync();
       int32_t total = 0;
-      for (int r = 0; r < kSoftCluster; ++r) total += sh.cnt[pass & 1][r];
-      if (total < top_k) lo_c = mid + 1;
-      else hi_c = mid;
+      for (int r = 0; r < K; ++r) total += sh.cnt[pass & 1][r];
+      if (total < top_k) {
+        lo_c = mid + 1;
+        step *= 2;
+      } else {
+        hi_c = mid;
+        out = true;
+      }
     }
     n_in = lo_c;
   }
@@ -680,6 +706,26 @@ __global__ void __cluster_dims__(kSoftCluster, 1, 1) __launch_bounds__(kSoftThre
   token_out[g] = tok;
   if (mass_out) mass_out[g] = soft ? mass : -1.f;
   mask_rows(s, row_active, g, rows_per_group);
+}
+
+// Clusters of K CTAs of the soft gate that the current device holds at once, asked
+// of the runtime once per device, logit type and K.
+cudaError_t soft_clusters(cudaLaunchConfig_t cfg, int32_t dtype, int K, int* out) {
+  constexpr int kMaxDev = 16;
+  static std::atomic<int> cache[kMaxDev][2][kSoftCluster + 1] = {};  // clusters + 1; 0: not asked yet
+  int dev = 0;
+  if (cudaError_t e = cudaGetDevice(&dev); e != cudaSuccess) return e;
+  std::atomic<int>* c = dev < kMaxDev ? &cache[dev][dtype == RGD_F32 ? 0 : 1][K] : nullptr;
+  if (const int n = c ? c->load(std::memory_order_relaxed) : 0; n > 0) {
+    *out = n - 1;
+    return cudaSuccess;
+  }
+  cfg.gridDim = dim3((unsigned)K);
+  cfg.numAttrs = 1;
+  const cudaError_t e = dtype == RGD_F32 ? cudaOccupancyMaxActiveClusters(out, soft_gate_kernel<float>, &cfg)
+                                         : cudaOccupancyMaxActiveClusters(out, soft_gate_kernel<uint16_t>, &cfg);
+  if (e == cudaSuccess && c) c->store(*out + 1, std::memory_order_relaxed);
+  return e;
 }
 
 }  // namespace
@@ -811,7 +857,7 @@ extern "C" int rgd_soft_gate(const rgd_trie* trie, int32_t groups, int32_t rows_
                              rgd_stream_t stream) {
   clear_error();
   RGD_CHECK_ARG(trie != nullptr, "rgd_soft_gate: trie is NULL");
-  RGD_CHECK_ARG(groups >= 0 && groups <= INT32_MAX / kSoftCluster && rows_per_group >= 1 && vocab >= 1,
+  RGD_CHECK_ARG(groups >= 0 && groups <= INT32_MAX / 6 && rows_per_group >= 1 && vocab >= 1,
                 "rgd_soft_gate: bad groups/rows/vocab");
   RGD_CHECK_ARG(dtype == RGD_F32 || dtype == RGD_BF16, "rgd_soft_gate: dtype must be RGD_F32 or RGD_BF16");
   RGD_CHECK_ARG(row_stride >= vocab, "rgd_soft_gate: row_stride < vocab");
@@ -833,14 +879,39 @@ extern "C" int rgd_soft_gate(const rgd_trie* trie, int32_t groups, int32_t rows_
     cudaFuncSetAttribute(soft_gate_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, kDyn);
     cudaFuncSetAttribute(soft_gate_kernel<uint16_t>, cudaFuncAttributeMaxDynamicSharedMemorySize, kDyn);
   });
+  cudaLaunchConfig_t cfg = {};
+  cfg.blockDim = dim3(kSoftThreads);
+  cfg.dynamicSmemBytes = kDyn;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  // CTAs per group: as many as let every group's cluster run at once (one CTA on an
+  // SM; clusters of 6 and 4 leave some of a processing cluster's SMs out): a second
+  // wave costs more than a longer share.  6 / 4 / 2 CTAs inside a graph, K = 40, 128256
+  // fp32 logits: 16 groups 13.7 / 16.1 / 23.7 us; 24 groups 19.7 / 16.3 / 23.7; 64
+  // groups 33.8 / 29.6 / 25.2; 200 groups of 32000 64 / 46 / 31 (1 CTA: 29).
+  int K = kSoftCluster;
+  cudaError_t e = cudaSuccess;
+  for (;; K -= 2) {
+    attr[0].val.clusterDim = {(unsigned)K, 1, 1};
+    if (K == 2) break;
+    int n = 0;
+    if ((e = soft_clusters(cfg, dtype, K, &n)) != cudaSuccess) return cuda_error(e, "soft_gate occupancy");
+    if (groups <= n) break;
+  }
+  cfg.gridDim = dim3((unsigned)(groups * K));
+  cfg.numAttrs = 2;
   if (dtype == RGD_F32)
-    soft_gate_kernel<float><<<groups * kSoftCluster, kSoftThreads, kDyn, st>>>(
-        tv, rows_per_group, vocab, static_cast<const float*>(probe_logits), row_stride, vec, top_k, rho, c, eos_token,
-        max_len, state, row_active, token_out, mass_out, dev_status);
+    e = cudaLaunchKernelEx(&cfg, soft_gate_kernel<float>, tv, rows_per_group, vocab,
+                           static_cast<const float*>(probe_logits), row_stride, vec, top_k, rho, c, eos_token, max_len,
+                           state, row_active, token_out, mass_out, dev_status);
   else
-    soft_gate_kernel<uint16_t><<<groups * kSoftCluster, kSoftThreads, kDyn, st>>>(
-        tv, rows_per_group, vocab, static_cast<const uint16_t*>(probe_logits), row_stride, vec, top_k, rho, c,
-        eos_token, max_len, state, row_active, token_out, mass_out, dev_status);
-  cudaError_t e = cudaGetLastError();
+    e = cudaLaunchKernelEx(&cfg, soft_gate_kernel<uint16_t>, tv, rows_per_group, vocab,
+                           static_cast<const uint16_t*>(probe_logits), row_stride, vec, top_k, rho, c, eos_token,
+                           max_len, state, row_active, token_out, mass_out, dev_status);
+  if (e == cudaSuccess) e = cudaGetLastError();
   return e == cudaSuccess ? RGD_OK : cuda_error(e, "soft_gate launch");
 }
