@@ -33,10 +33,10 @@ inline int align_up(int x, int a) { return (x + a - 1) / a * a; }
 // 32 queries; then three or four sets of 16, 24 or 32, the smallest that holds
 // the count, since the MMAs' columns and the P^T writes go with sets x per_set.
 // Per query count (us; 64 or 32 query heads, 8 kv heads), against a kernel that
-// held 128 rows of query copies whatever the count: 12 in (2, 8): 56 (73 with
-// copies), 16: 65 (82), 32 in (4, 8): 65 (75), 36 in (3, 16): 51 (70), 56 in
-// (4, 16): 76 (100), 72 in (3, 24): 120 (202), 96 in (4, 24): 103 (138), 128 in
-// (4, 32): 134 (150).
+// held 128 rows of query copies whatever the count: 12 in (2, 8): 54 (73 with
+// copies), 16: 62 (82), 32 in (4, 8): 57 (75), 36 in (3, 16): 47 (70), 56 in
+// (4, 16): 71 (100), 72 in (3, 24): 115 (202), 96 in (4, 24): 92 (138), 128 in
+// (4, 32): 121 (150).
 struct QueryConfig {
   int sets, per_set;
 };

@@ -50,8 +50,8 @@
 //   16 x 5, 32/8, 128, 512-2048                                     36 -> 29.5
 //   1 x 5, 32/8, 128, 3000                                          25 -> 15.3
 //   12 x 9, 32/8, 128, 500-6000                                     70 -> 47
-//   4 x 9, 64/8, 128, 32768                                        202 -> 118
-//   32 x 16, 64/8, 128, 200-800                                    107 -> 83
+//   4 x 9, 64/8, 128, 32768                                        202 -> 115
+//   32 x 16, 64/8, 128, 200-800                                    107 -> 82
 //   200 x 16, 4/1, 64, 50-100                                       35 -> 32
 // Every wait on an mbarrier is bounded; a timeout is reported in the status
 // word and every role stops.
@@ -331,14 +331,37 @@ __device__ __forceinline__ float transpose_reduce8(float (&v)[8], int lane, Op o
   return v[0];
 }
 
+// Two fp32 values in one 64-bit register, and a fused multiply-add or a sum of both
+// at once (a softmax thread's arithmetic is all in pairs: half the issue slots).
+__device__ __forceinline__ uint64_t pair(float a, float b) {
+  uint64_t r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ float2 unpair(uint64_t a) {
+  float2 r;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(a));
+  return r;
+}
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
+  uint64_t r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
 // P = hi + lo with hi = p truncated to bf16 and lo = (p - hi) truncated to bf16
 // (|p - hi - lo| <= 2^-16 |p|), two values per 32-bit word, the first in the
 // low half.
 __device__ __forceinline__ void split_bf16x2(float p0, float p1, uint32_t& hi, uint32_t& lo) {
-  const uint32_t h0 = __float_as_uint(p0) & 0xffff0000u, h1 = __float_as_uint(p1) & 0xffff0000u;
-  const uint32_t l0 = __float_as_uint(p0 - __uint_as_float(h0)), l1 = __float_as_uint(p1 - __uint_as_float(h1));
-  hi = (h0 >> 16) | h1;
-  lo = (l0 >> 16) | (l1 & 0xffff0000u);
+  const uint32_t u0 = __float_as_uint(p0), u1 = __float_as_uint(p1);
+  const uint64_t h = pair(__uint_as_float(u0 & 0xffff0000u), __uint_as_float(u1 & 0xffff0000u));
+  const float2 l = unpair(fma2(h, pair(-1.f, -1.f), pair(p0, p1)));  // (exact)
+  hi = __byte_perm(u0, u1, 0x7632);
+  lo = __byte_perm(__float_as_uint(l.x), __float_as_uint(l.y), 0x7632);
 }
 
 // The merge of a split job by every warp of the block that holds its first page,
@@ -1023,9 +1046,10 @@ __global__ void __launch_bounds__(AttnCfg<D, NS, QS>::kThreads, 1)
       if (hi <= lo) return 0u;
       return (hi - lo >= 32 ? 0xffffffffu : ((1u << (hi - lo)) - 1u)) << lo;
     };
-    float lacc[QS];
+    uint64_t lacc[QS / 2];  // (pairs)
 #pragma unroll
-    for (int i = 0; i < QS; ++i) lacc[i] = 0.f;
+    for (int i = 0; i < QS / 2; ++i) lacc[i] = 0;
+    const uint64_t scale2 = pair(p.scale_log2, p.scale_log2);
     int mv = 0;         // current version of the reference maxima
     bool fresh = true;  // piece start: every reference is -inf (not read from shared memory)
     int gi = 0;
@@ -1069,10 +1093,10 @@ __global__ void __launch_bounds__(AttnCfg<D, NS, QS>::kThreads, 1)
 #pragma unroll
             for (int q = 0; q < 8; q += 4) {
               const float4 n4 = fresh ? make_float4(kNoRef, kNoRef, kNoRef, kNoRef) : *reinterpret_cast<const float4*>(nr + q);
-              mx = fmaxf(fmaxf(mx, fmaf(__uint_as_float(x[q]), p.scale_log2, n4.x)),
-                         fmaf(__uint_as_float(x[q + 1]), p.scale_log2, n4.y));
-              mx = fmaxf(fmaxf(mx, fmaf(__uint_as_float(x[q + 2]), p.scale_log2, n4.z)),
-                         fmaf(__uint_as_float(x[q + 3]), p.scale_log2, n4.w));
+              const float2 a = unpair(fma2(pair(__uint_as_float(x[q]), __uint_as_float(x[q + 1])), scale2, pair(n4.x, n4.y)));
+              const float2 c2 = unpair(fma2(pair(__uint_as_float(x[q + 2]), __uint_as_float(x[q + 3])), scale2, pair(n4.z, n4.w)));
+              mx = fmaxf(fmaxf(mx, a.x), a.y);
+              mx = fmaxf(fmaxf(mx, c2.x), c2.y);
             }
           };
           if (QS <= 16) {  // the scores stay in registers
@@ -1121,7 +1145,10 @@ __global__ void __launch_bounds__(AttnCfg<D, NS, QS>::kThreads, 1)
             const float fq = mo == -INFINITY ? 0.f : exp2f(mo - mn);
             if (qd == 0 && lane < QS) nref[(mv ^ 1) * C::kNq + qi] = mn == -INFINITY ? kNoRef : -mn;
 #pragma unroll
-            for (int q = 0; q < QS; ++q) lacc[q] *= __shfl_sync(0xffffffffu, fq, q);
+            for (int q = 0; q < QS; q += 2) {
+              const float2 l = unpair(lacc[q / 2]);
+              lacc[q / 2] = pair(l.x * __shfl_sync(0xffffffffu, fq, q), l.y * __shfl_sync(0xffffffffu, fq, q + 1));
+            }
             // O^T already holds this piece's earlier groups: once their PV is
             // done, the set's query columns (this warp's 32 head dimensions) are scaled
             if (k0 > 0) {
@@ -1173,14 +1200,13 @@ __global__ void __launch_bounds__(AttnCfg<D, NS, QS>::kThreads, 1)
 #pragma unroll
               for (int q = 0; q < 8; q += 4) {
                 const float4 n4 = fresh ? make_float4(0.f, 0.f, 0.f, 0.f) : *reinterpret_cast<const float4*>(nr + q);
-                const float nn[4] = {n4.x, n4.y, n4.z, n4.w};
+                const uint64_t nn[2] = {pair(n4.x, n4.y), pair(n4.z, n4.w)};
 #pragma unroll
                 for (int u = 0; u < 4; u += 2) {
                   const int i = q + u;
-                  const float p0 = ex2_approx(fmaf(__uint_as_float(x[i]), p.scale_log2, nn[u]));
-                  const float p1 = ex2_approx(fmaf(__uint_as_float(x[i + 1]), p.scale_log2, nn[u + 1]));
-                  lacc[ch * 8 + i] += p0;
-                  lacc[ch * 8 + i + 1] += p1;
+                  const float2 t2 = unpair(fma2(pair(__uint_as_float(x[i]), __uint_as_float(x[i + 1])), scale2, nn[u / 2]));
+                  const float p0 = ex2_approx(t2.x), p1 = ex2_approx(t2.y);
+                  lacc[(ch * 8 + i) / 2] = add2(lacc[(ch * 8 + i) / 2], pair(p0, p1));
                   split_bf16x2(p0, p1, hi[i / 2], lo[i / 2]);
                 }
               }
@@ -1207,9 +1233,11 @@ __global__ void __launch_bounds__(AttnCfg<D, NS, QS>::kThreads, 1)
         for (int ch = 0; ch < kCh; ++ch) {
           float v[8];
 #pragma unroll
-          for (int q = 0; q < 8; ++q) {
-            v[q] = lacc[ch * 8 + q];
-            lacc[ch * 8 + q] = 0.f;
+          for (int q = 0; q < 8; q += 2) {
+            const float2 l = unpair(lacc[(ch * 8 + q) / 2]);
+            v[q] = l.x;
+            v[q + 1] = l.y;
+            lacc[(ch * 8 + q) / 2] = 0;
           }
           const float ls = transpose_reduce8(v, lane, [](float x, float y) { return x + y; });
           if (lane < 8) {
