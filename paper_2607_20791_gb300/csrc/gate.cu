@@ -473,7 +473,7 @@ __global__ void __launch_bounds__(kSoftThreads, 1)
   const float p_min = np_ > 0 ? pv[np_ - 1] : INFINITY;  // only a logit >= this can rank above a probe
 
   // ---- the pass: maximum, its lowest index, z = sum e^(l - m), probe ranks ----
-  float m = -INFINITY, z = 0.f;
+  float m = -INFINITY, z = 0.f, z_lo = 0.f;  // (z_lo: what the sums of the chunks' shares round off)
   int32_t mi = 0x7fffffff;
   auto probe_counts = [&](float v, int32_t i) {
 #pragma unroll
@@ -511,7 +511,9 @@ __global__ void __launch_bounds__(kSoftThreads, 1)
           for (int e = E - 1; e >= 0; --e)
             if (vec_elem<LT>(x, e) == bm) bi = (base + k) * E + e;
         }
-        z = (m == -INFINITY) ? 0.f : z * ex2_approx((m - bm) * kLog2e);
+        const float f = m == -INFINITY ? 0.f : ex2_approx((m - bm) * kLog2e);
+        z *= f;
+        z_lo *= f;
         m = bm;
         mi = bi;
       }
@@ -533,7 +535,9 @@ __global__ void __launch_bounds__(kSoftThreads, 1)
           }
           zc += z0 + z1;
         }
-        z += zc;
+        const float sum = z + zc, up = sum - z;
+        z_lo += (z - (sum - up)) + (zc - up);
+        z = sum;
       } else if (bm >= p_min) {  // (every logit so far is -inf, and so is a probed candidate)
 #pragma unroll 1
         for (int32_t k = tid; k < cnt; k += kSoftThreads) {
@@ -547,6 +551,7 @@ __global__ void __launch_bounds__(kSoftThreads, 1)
         if (tid == 0) issue(ck + kSoftStages);
       }
     }
+    z += z_lo;
     // the few logits past the last whole vector
     const int32_t i = nvec * E + tid;
     if (rank == K - 1 && i < vocab) one(logit_at<LT>(row, i), i);
