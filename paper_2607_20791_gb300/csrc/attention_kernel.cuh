@@ -830,55 +830,54 @@ __global__ void __launch_bounds__(AttnCfg<D, NS, QS>::kThreads, 1)
     const uint64_t pol = policy_evict_first();
     const int n_pages = e - b;
     int gbase = 0;  // groups started before sequence position ib
-    PageRef nxt{};
+    PageRef nxt = resolve_page(ctx, lane);
 #pragma unroll 1
-    for (int ib = -32; ib < n_pages; ib += 32) {
+    for (int ib = 0; ib < n_pages; ib += 32) {
       const PageRef cur = nxt;
       bool have_next = false;
-      if (ib >= 0) {
-        const bool valid = ib + lane < n_pages;
-        const bool start = valid && cur.pos == 0;
-        const uint32_t starts = __ballot_sync(0xffffffffu, start);
-        const uint32_t le = 0xffffffffu >> (31 - lane);
-        const int gidx = gbase + __popc(starts & le) - 1;  // lane 0 may continue the last round's group
-        const int g0 = __shfl_sync(0xffffffffu, gidx, 0);
-        const int g1 = __shfl_sync(0xffffffffu, gidx, 31 - __clz(__ballot_sync(0xffffffffu, valid)));
-        gbase += __popc(starts);
-        const int gs = gidx - (int)(((uint64_t)(uint32_t)gidx * nr_mul) >> 32) * nr;  // gidx % nr
-        bool aborted = false;
+      const bool valid = ib + lane < n_pages;
+      const bool start = valid && cur.pos == 0;
+      const uint32_t starts = __ballot_sync(0xffffffffu, start);
+      const uint32_t le = 0xffffffffu >> (31 - lane);
+      const int gidx = gbase + __popc(starts & le) - 1;  // lane 0 may continue the last round's group
+      const int g0 = __shfl_sync(0xffffffffu, gidx, 0);
+      const int g1 = __shfl_sync(0xffffffffu, gidx, 31 - __clz(__ballot_sync(0xffffffffu, valid)));
+      gbase += __popc(starts);
+      const int gs = gidx - (int)(((uint64_t)(uint32_t)gidx * nr_mul) >> 32) * nr;  // gidx % nr
+      bool aborted = false;
 #pragma unroll 1
-        for (int gq = g0; gq <= g1; ++gq) {
-          if (gq >= nr) {
-            if (!have_next && ib + 32 < n_pages) {
-              nxt = resolve_page(ctx, ib + 32 + lane);
-              have_next = true;
-            }
-            const bool ok = wait_or_abort(&empty[gq % nr], (uint32_t)((gq / nr) - 1) & 1u, abort_flag, p.wait_ns);
-            if (!__all_sync(0xffffffffu, ok)) {
-              aborted = true;
-              break;
-            }
+      for (int gq = g0; gq <= g1; ++gq) {
+        if (gq >= nr) {
+          if (!have_next && ib + 32 < n_pages) {
+            nxt = resolve_page(ctx, ib + 32 + lane);
+            have_next = true;
           }
-          if (valid && gidx == gq) {
-            int32_t y = -2 * kPage;  // fully out of bounds: the TMA fills zeros
-            if (cur.page >= 0 && cur.page < p.num_pages) y = (cur.page * p.Hkv + cur.h) * kPage;
-            else flag(p.dev_status, RGD_DEV_BAD_PAGE);
-            uint8_t* sl = ring + gs * C::kArea;
-            mbar_arrive_expect_tx(&full[gs], kTile);
-            if (is_v) {
-              tma_load_3d_hint(sl + cur.pos * kTile, &tmV, &full[gs], 0, y, 0, pol);
-            } else {
-              descs[(gq & 7) * kGroupPages + cur.pos] = cur.desc;
-#pragma unroll
-              for (int hf = 0; hf < kHalves; ++hf)
-                tma_load_3d_hint(sl + hf * (kGroupPages * 2048) + cur.pos * 2048, &tmK, &full[gs], 0, y, hf, pol);
-            }
-            if (cur.pos == cur.ng - 1 && cur.ng < kGroupPages) mbar_arrive_cnt(&full[gs], kGroupPages - cur.ng);
-            if (start) atomicMax(&s_issued[is_v], gq + 1);
+          const int use = (int)(((uint64_t)(uint32_t)gq * nr_mul) >> 32);  // gq / nr
+          const bool ok = wait_or_abort(&empty[gq - use * nr], (uint32_t)(use - 1) & 1u, abort_flag, p.wait_ns);
+          if (!__all_sync(0xffffffffu, ok)) {
+            aborted = true;
+            break;
           }
         }
-        if (aborted) break;
+        if (valid && gidx == gq) {
+          int32_t y = -2 * kPage;  // fully out of bounds: the TMA fills zeros
+          if (cur.page >= 0 && cur.page < p.num_pages) y = (cur.page * p.Hkv + cur.h) * kPage;
+          else flag(p.dev_status, RGD_DEV_BAD_PAGE);
+          uint8_t* sl = ring + gs * C::kArea;
+          mbar_arrive_expect_tx(&full[gs], kTile);
+          if (is_v) {
+            tma_load_3d_hint(sl + cur.pos * kTile, &tmV, &full[gs], 0, y, 0, pol);
+          } else {
+            descs[(gq & 7) * kGroupPages + cur.pos] = cur.desc;
+#pragma unroll
+            for (int hf = 0; hf < kHalves; ++hf)
+              tma_load_3d_hint(sl + hf * (kGroupPages * 2048) + cur.pos * 2048, &tmK, &full[gs], 0, y, hf, pol);
+          }
+          if (cur.pos == cur.ng - 1 && cur.ng < kGroupPages) mbar_arrive_cnt(&full[gs], kGroupPages - cur.ng);
+          if (start) atomicMax(&s_issued[is_v], gq + 1);
+        }
       }
+      if (aborted) break;
       if (!have_next && ib + 32 < n_pages) nxt = resolve_page(ctx, ib + 32 + lane);
       __syncwarp();
     }
