@@ -30,19 +30,25 @@ PFN_cuTensorMapEncodeTiled_v12000 get_encode_fn() {
   return fn;
 }
 
-int make_kv_map(CUtensorMap* map, const void* base, int64_t rows, int D, int box_halves) {
+// The K or V pool ([rows][D] bf16) for copies of whole 16-token page-head tiles, one
+// box each, with the 128-byte swizzle (16-byte chunk index XOR row index mod 8).
+// V: 64 columns x 16 rows x D/64 halves, so a tile lands half-major.  K: 64 columns x
+// 8 rows x D/64 halves x 2 row groups, so that consecutive 8-row groups of a half
+// are D/64 KB apart within a tile and across tiles: a group's K is one 128-row
+// operand per half although each page is one box (with a box per half the K
+// producer's issue, ~75 cycles a box, was twice the V producer's).
+int make_kv_map(CUtensorMap* map, const void* base, int64_t rows, int D, bool is_k) {
   auto fn = get_encode_fn();
   if (!fn) return set_error(RGD_ERR_CUDA, "cuTensorMapEncodeTiled is unavailable");
-  // View each 16-token page-head tile as (64 columns) x (16 rows) x (D/64 halves):
-  // a box is one half or the whole tile, laid out in shared memory half-major
-  // with the 128-byte swizzle (16-byte chunk index XOR row index mod 8).
-  cuuint64_t dims[3] = {64, (cuuint64_t)rows, (cuuint64_t)(D / 64)};
-  cuuint64_t strides[2] = {(cuuint64_t)D * 2, 128};
-  cuuint32_t box[3] = {64, (cuuint32_t)kPage, (cuuint32_t)box_halves};
-  cuuint32_t estr[3] = {1, 1, 1};
-  CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, estr,
-                  CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                  CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  const cuuint32_t halves = (cuuint32_t)(D / 64);
+  const cuuint64_t row = (cuuint64_t)D * 2;
+  const cuuint64_t dims_k[4] = {64, 8, halves, (cuuint64_t)rows / 8}, strides_k[3] = {row, 128, 8 * row};
+  const cuuint64_t dims_v[3] = {64, (cuuint64_t)rows, halves}, strides_v[2] = {row, 128};
+  const cuuint32_t box_k[4] = {64, 8, halves, kPage / 8}, box_v[3] = {64, (cuuint32_t)kPage, halves};
+  const cuuint32_t estr[4] = {1, 1, 1, 1};
+  CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, is_k ? 4 : 3, const_cast<void*>(base), is_k ? dims_k : dims_v,
+                  is_k ? strides_k : strides_v, is_k ? box_k : box_v, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                  CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   if (r != CUDA_SUCCESS) return set_error(RGD_ERR_CUDA, "cuTensorMapEncodeTiled failed (%d)", (int)r);
   return RGD_OK;
 }
@@ -187,8 +193,8 @@ extern "C" int rgd_prefix_decode_attn(const rgd_attn_shape* shape, const rgd_bf1
 
   CUtensorMap tmK, tmV;
   const int64_t kv_rows = (int64_t)s.num_pages * s.num_kv_heads * kPage;
-  if (int rc = make_kv_map(&tmK, k_pages, kv_rows, s.head_dim, 1)) return rc;                // one half per box
-  if (int rc = make_kv_map(&tmV, v_pages, kv_rows, s.head_dim, s.head_dim / 64)) return rc;  // whole tile
+  if (int rc = make_kv_map(&tmK, k_pages, kv_rows, s.head_dim, true)) return rc;
+  if (int rc = make_kv_map(&tmV, v_pages, kv_rows, s.head_dim, false)) return rc;
 
   AttnParams p;
   p.q = reinterpret_cast<const __nv_bfloat16*>(q);

@@ -63,7 +63,7 @@ inline AttnLayout attn_layout(int D, int sets, int per_set, int hk, int hv, int 
                               bool slen_in_smem) {
   const int area = kGroupPages * kPage * D * 2, N = query_cols(sets, per_set), nq = sets * per_set;
   AttnLayout L;
-  L.kring = 0;                                // [hk][D/64 halves][8 pages][16 rows][128 B]
+  L.kring = 0;                                // [hk][8 pages][2 row groups][D/64 halves][8 rows][128 B]
   L.vring = L.kring + hk * area;              // [hv][8 pages][D/64 halves][16 rows][128 B]
   L.p = L.vring + hv * area;                  // [np] P^T: 128 tokens x (N high parts, N residuals) bf16
   L.q = L.p + np * 512 * N;                   // [nqb][D/64 halves][N rows][128 B]

@@ -46,12 +46,12 @@
 // -> block table -> data) and the merge at the end.  Measured inside a CUDA
 // graph, against a kernel with the queries as the MMA's M (128 rows of query
 // copies), P in tensor memory and one ring for K and V together (us):
-//   256 groups x 2 rows, 32/8 heads, D 128, prompts of 128-8192    440 -> 355 (0.97 of the copy rate)
-//   16 x 5, 32/8, 128, 512-2048                                     36 -> 29.5
-//   1 x 5, 32/8, 128, 3000                                          25 -> 15.3
-//   12 x 9, 32/8, 128, 500-6000                                     70 -> 47
-//   4 x 9, 64/8, 128, 32768                                        202 -> 115
-//   32 x 16, 64/8, 128, 200-800                                    107 -> 82
+//   256 groups x 2 rows, 32/8 heads, D 128, prompts of 128-8192    440 -> 353 (0.98 of the copy rate)
+//   16 x 5, 32/8, 128, 512-2048                                     36 -> 29
+//   1 x 5, 32/8, 128, 3000                                          25 -> 15.0
+//   12 x 9, 32/8, 128, 500-6000                                     70 -> 46
+//   4 x 9, 64/8, 128, 32768                                        202 -> 114
+//   32 x 16, 64/8, 128, 200-800                                    107 -> 81
 //   200 x 16, 4/1, 64, 50-100                                       35 -> 32
 // Every wait on an mbarrier is bounded; a timeout is reported in the status
 // word and every role stops.
@@ -815,10 +815,10 @@ __global__ void __launch_bounds__(AttnCfg<D, NS, QS>::kThreads, 1)
 
   if (warp == C::kProdK || warp == C::kProdV) {
     // ============================ producers ===========================
-    // One warp for K and one for V, 32 pages (one per lane) a round, groups of 8
-    // pages; an issuing lane's copies take ~75 cycles each, hence two warps.  A
-    // group's K lands half-major ([D/64][8 pages][16 rows][128 B], so that it is
-    // one 128-row A operand per half), V tiles page-major.  The next round's pages
+    // One warp for K and one for V, 32 pages (one per lane, one copy each) a round,
+    // groups of 8 pages; a copy takes its issuer ~75 cycles, hence two warps.  A K
+    // tile lands as [2 row groups][D/64][8 rows][128 B], so that a group is one
+    // 128-row A operand per half, a V tile as [D/64][16 rows][128 B].  The next round's pages
     // are resolved (job by binary search, then the block-table entry) before the
     // first wait of a round, so the block-table loads are in flight meanwhile.
     const bool is_v = warp == C::kProdV;
@@ -869,9 +869,7 @@ __global__ void __launch_bounds__(AttnCfg<D, NS, QS>::kThreads, 1)
             tma_load_3d_hint(sl + cur.pos * kTile, &tmV, &full[gs], 0, y, 0, pol);
           } else {
             descs[(gq & 7) * kGroupPages + cur.pos] = cur.desc;
-#pragma unroll
-            for (int hf = 0; hf < kHalves; ++hf)
-              tma_load_3d_hint(sl + hf * (kGroupPages * 2048) + cur.pos * 2048, &tmK, &full[gs], 0, y, hf, pol);
+            tma_load_4d_hint(sl + cur.pos * kTile, &tmK, &full[gs], 0, 0, 0, y / 8, pol);
           }
           if (cur.pos == cur.ng - 1 && cur.ng < kGroupPages) mbar_arrive_cnt(&full[gs], kGroupPages - cur.ng);
           if (start) atomicMax(&s_issued[is_v], gq + 1);
@@ -921,7 +919,7 @@ __global__ void __launch_bounds__(AttnCfg<D, NS, QS>::kThreads, 1)
   } else if (warp == C::kQk) {
     // ============================ QK issue ============================
     if (lane == 0 && b < e) {
-      const uint64_t kdesc = smem_desc(sbase + L.kring, 16, 1024, 2);
+      const uint64_t kdesc = smem_desc(sbase + L.kring, 16, kHalves * 1024, 2);
       const uint64_t qdesc = smem_desc(sbase + L.q, 16, 1024, 2);
       int gi = 0, pc = 0, gs = 0;
       uint32_t ph = 0;
@@ -943,7 +941,7 @@ __global__ void __launch_bounds__(AttnCfg<D, NS, QS>::kThreads, 1)
           tc_fence_after();
           uint64_t a = kdesc + (uint64_t)((gs * C::kArea) >> 4), bq = qdesc + (uint64_t)((qb * C::kQBytes) >> 4);
 #pragma unroll 1
-          for (int hf = 0; hf < kHalves; ++hf, a += kGroupPages * 2048 >> 4, bq += C::kN * 128 >> 4) {
+          for (int hf = 0; hf < kHalves; ++hf, a += 1024 >> 4, bq += C::kN * 128 >> 4) {
 #pragma unroll
             for (int kk = 0; kk < 4; ++kk)  // 16 of the half's 64 columns
               umma_bf16(tmem + C::kSCol + sb * C::kN, a + kk * 2, bq + kk * 2, kIdQK, (hf | kk) != 0 ? 1u : 0u);
