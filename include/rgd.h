@@ -27,6 +27,10 @@
  *     the shapes given, and 16-byte aligned base addresses.
  *   - Calls are asynchronous on `stream` (a cudaStream_t; NULL = the legacy
  *     default stream) and use the device that is current on the calling thread.
+ *     Their kernels are launched as programmatic dependents of the previous
+ *     kernel on the stream: they are scheduled while it finishes and wait for it
+ *     before they read or write anything (the head inside rgd_decode_step reads
+ *     its inputs, complete by then, while the step's attention runs).
  *   - The return value is a host status: RGD_OK, or an RGD_ERR_* code when the
  *     arguments are rejected (nothing is launched) or a launch fails;
  *     rgd_last_error_string() then describes the error (per thread).
@@ -344,8 +348,8 @@ int rgd_decode_step(const rgd_attn_shape* shape, const rgd_bf16* q, const rgd_bf
  * be NULL) gets RGD_DEV_WAIT_TIMEOUT when a bounded wait on a copy of the
  * logits gave up; that step's outputs are then not valid.
  * RGD_ERR_UNSUPPORTED when a trie node has more than 2047 children.  One
- * kernel on `stream`: a cluster of 6 blocks per group, each block reading a
- * sixth of the probe row. */
+ * kernel on `stream`: a cluster of 6, 4 or 2 blocks per group, each block reading
+ * an equal share of the probe row. */
 int rgd_soft_gate(const rgd_trie* trie, int32_t groups, int32_t rows_per_group, int32_t vocab, int32_t dtype,
                   const void* probe_logits, int64_t row_stride, int32_t top_k, float rho, int32_t c,
                   int32_t eos_token, int32_t max_len, rgd_gate_state* state, uint8_t* row_active,
