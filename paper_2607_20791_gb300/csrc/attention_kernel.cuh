@@ -864,13 +864,11 @@ __global__ void __launch_bounds__(AttnCfg<D, NS, QS>::kThreads, 1)
           if (cur.page >= 0 && cur.page < p.num_pages) y = (cur.page * p.Hkv + cur.h) * kPage;
           else flag(p.dev_status, RGD_DEV_BAD_PAGE);
           uint8_t* sl = ring + gs * C::kArea;
+          // (the descriptor before the arrival, which releases it to the QK thread and so to the softmax)
+          if (!is_v) descs[(gq & 7) * kGroupPages + cur.pos] = cur.desc;
           mbar_arrive_expect_tx(&full[gs], kTile);
-          if (is_v) {
-            tma_load_3d_hint(sl + cur.pos * kTile, &tmV, &full[gs], 0, y, 0, pol);
-          } else {
-            descs[(gq & 7) * kGroupPages + cur.pos] = cur.desc;
-            tma_load_4d_hint(sl + cur.pos * kTile, &tmK, &full[gs], 0, 0, 0, y / 8, pol);
-          }
+          if (is_v) tma_load_3d_hint(sl + cur.pos * kTile, &tmV, &full[gs], 0, y, 0, pol);
+          else tma_load_4d_hint(sl + cur.pos * kTile, &tmK, &full[gs], 0, 0, 0, y / 8, pol);
           if (cur.pos == cur.ng - 1 && cur.ng < kGroupPages) mbar_arrive_cnt(&full[gs], kGroupPages - cur.ng);
           if (start) atomicMax(&s_issued[is_v], gq + 1);
         }
