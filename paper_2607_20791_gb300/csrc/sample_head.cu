@@ -575,8 +575,13 @@ __global__ void __launch_bounds__(kHeadThreads, 3) sample_head_kernel(const Head
   // Round k gives the cluster row k * stride + (cid + k) % stride: shifted by
   // one each round, so that no cluster is left with one kind of row only where
   // the kinds repeat (probes and samples, temperatures).  Every warp takes the
-  // rounds in blocks of 32, lane k % 32 reading round k's activity (a row's flag
-  // does not change before every warp of its cluster is done with the row).
+  // rounds in blocks of 32, lane k % 32 reading round k's activity.  The gate may
+  // clear the flag of an active row once the row is finished, by CTA 0's draw warp
+  // alone if it is greedy, so every warp of the cluster must have read the block's
+  // flags by then.  It has: a row is finished behind the exchange of its maxima, to
+  // which every stream warp of the cluster contributes only after its own copy warp's
+  // copies and its own draw warp's parameters of the block, and both of these read
+  // the flags first.
   const int nblk = ((p.rows + stride - 1) / stride + 31) / 32;
   auto row_of = [&](int k) { return k * stride + (cid + k) % stride; };
   auto block_rows = [&](int blk) {
@@ -857,11 +862,15 @@ __global__ void __launch_bounds__(kHeadThreads, 3) sample_head_kernel(const Head
   } else {
     // ============================== draw warp ==============================
     asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-    // The parameters of a block's 32 rows, one lane each: the min-p offset
-    // T ln p_min (fp64 logarithm) and the draw's uniform.
+    // The active rows of a block, and the parameters of its 32 rows, one lane each:
+    // the min-p offset T ln p_min (fp64 logarithm) and the draw's uniform.  The
+    // arrival that publishes the parameters comes after the flags have been read
+    // (see above; read behind it, a flag could already be this launch's gate's).
     auto fill = [&](int blk) {
-      if (blk >= nblk) return;
+      if (blk >= nblk) return 0u;
       const int row = row_of(blk * 32 + lane);
+      bool active = row < p.rows;
+      if (active && p.row_active) active = p.row_active[row] != 0;
       if (row < p.rows) {
         const float temp = p.temperature[row], mp = p.min_p[row];
         const bool greedy = (p.is_probe && p.is_probe[row]) || temp == 0.0f;
@@ -877,15 +886,17 @@ __global__ void __launch_bounds__(kHeadThreads, 3) sample_head_kernel(const Head
         rp.valid = temp >= 0.0f && isfinite(temp) && mp >= 0.0f && mp <= 1.0f;
         sh.prm[blk & 1][lane] = rp;
       }
+      const uint32_t rows = __ballot_sync(0xffffffffu, active);
       __syncwarp();
       if (lane == 0) mbar_arrive(&sh.prm_bar[blk & 1]);
+      return rows;
     };
-    fill(0);
+    uint32_t next_rows = fill(0);
     if (p.early) asm volatile("griddepcontrol.wait;" ::: "memory");
     int it = 0, xc = 0;  // rows, and exchanges of weight sums, so far
     for (int blk = 0; blk < nblk; ++blk) {
-      uint32_t mask_rows32 = block_rows(blk);
-      fill(blk + 1);  // (over the parameters of block blk - 1, which every warp is done with)
+      uint32_t mask_rows32 = next_rows;
+      next_rows = fill(blk + 1);  // (over the parameters of block blk - 1, which every warp is done with)
       if (rank == 0) {  // the block's inactive rows
         const int r = row_of(blk * 32 + lane);
         if (r < p.rows && !((mask_rows32 >> lane) & 1u)) {
