@@ -329,13 +329,13 @@ struct Shared {
   int32_t wcnt[2][kHeadWarps];
   float row_max[2];
   int32_t row_arg[2];
-  RowParams prm[2][32];  // a block of the cluster's rows: the draw warp -> the stream warps
+  RowParams prm[2][32];  // a block of the cluster's rows with an active one: the draw warp -> the stream warps
   uint64_t full_bar[kMaxSlots];   // a ring slot's copy has landed
   uint64_t empty_bar[kMaxSlots];  // every stream warp is done with the slot
   uint64_t max_bar[2];   // every warp's max is in wmax
   uint64_t sum_bar[2];   // this CTA's stream warps are done with the row
   uint64_t csum_bar[2];  // every CTA's sum is in csum
-  uint64_t prm_bar[2];   // the block's parameters are in place
+  uint64_t prm_bar[2];   // the block's parameters are in place (blocks without an active row have no phase)
   uint64_t free_bar[2];  // the draw warp is done with the row
   int32_t abort;         // a wait gave up: every later wait returns at once
 };
@@ -650,18 +650,19 @@ __global__ void __launch_bounds__(kHeadThreads, 3) sample_head_kernel(const Head
     int vend = kAligned ? min(p.vocab / kN, c0 + p.cvec) : 0, safe_lo = 0, safe_hi = vend;
     int pos = 0;
     uint32_t phase = 0;  // ring position of the next slot, and its phase
-    int it = 0;
+    int it = 0, nb = -1;  // rows so far, and the block's number among those with an active row
     for (int blk = 0; blk < nblk; ++blk) {
       uint32_t mask_rows32 = block_rows(blk);
+      nb += mask_rows32 != 0 ? 1 : 0;
       bool have_prm = false;
-      auto block_params = [&]() {  // (waited for in every block, so that no phase is missed)
-        if (!have_prm) wait(&sh.prm_bar[blk & 1], (uint32_t)(blk >> 1) & 1u, false);
+      auto block_params = [&]() {  // (by the block's first row)
+        if (!have_prm) wait(&sh.prm_bar[nb & 1], (uint32_t)(nb >> 1) & 1u, false);
         have_prm = true;
       };
       for (; mask_rows32; mask_rows32 &= mask_rows32 - 1, ++it) {
         const int kk = __ffs(mask_rows32) - 1;
         const int row = row_of(blk * 32 + kk);
-        const RowParams& rp = sh.prm[blk & 1][kk];
+        const RowParams& rp = sh.prm[nb & 1][kk];
         const int buf = it & 1;
         const uint32_t par = (uint32_t)(it >> 1) & 1u;
         RowView rv;
@@ -857,7 +858,6 @@ __global__ void __launch_bounds__(kHeadThreads, 3) sample_head_kernel(const Head
         __syncwarp();
         if (lane == 0) mbar_arrive(&sh.sum_bar[buf]);
       }
-      block_params();
     }
   } else {
     // ============================== draw warp ==============================
@@ -866,16 +866,24 @@ __global__ void __launch_bounds__(kHeadThreads, 3) sample_head_kernel(const Head
     // the min-p offset T ln p_min (fp64 logarithm) and the draw's uniform.  The
     // arrival that publishes the parameters comes after the flags have been read
     // (see above; read behind it, a flag could already be this launch's gate's).
+    // Only blocks with an active row take a parameter buffer and a phase of prm_bar:
+    // every stream warp waits for the phase before the block's first row counts as
+    // summed, and this warp is through with a block's rows before it fills the
+    // second block after it, so no phase is passed and no buffer overwritten early.
+    // (In a block without an active row this warp waits for nothing; were it to
+    // publish there, it could run ahead of a stream warp by two phases of one
+    // barrier, which that warp could not tell from none.)
+    int filled = 0;
     auto fill = [&](int blk) {
       if (blk >= nblk) return 0u;
       const int row = row_of(blk * 32 + lane);
       bool active = row < p.rows;
       if (active && p.row_active) active = p.row_active[row] != 0;
+      RowParams rp{};
       if (row < p.rows) {
         const float temp = p.temperature[row], mp = p.min_p[row];
         const bool greedy = (p.is_probe && p.is_probe[row]) || temp == 0.0f;
         const uint64_t sd = p.seed[row];
-        RowParams rp;
         rp.theta = -INFINITY;
         if (mp > 0.0f && !greedy) rp.theta = (float)((double)temp * log((double)mp));
         rp.kexp = 1.4426950408889634f / temp;
@@ -884,19 +892,22 @@ __global__ void __launch_bounds__(kHeadThreads, 3) sample_head_kernel(const Head
         rp.u24 = x0 >> 8;
         rp.greedy = greedy;
         rp.valid = temp >= 0.0f && isfinite(temp) && mp >= 0.0f && mp <= 1.0f;
-        sh.prm[blk & 1][lane] = rp;
       }
       const uint32_t rows = __ballot_sync(0xffffffffu, active);
+      if (rows == 0) return 0u;
+      sh.prm[filled & 1][lane] = rp;
       __syncwarp();
-      if (lane == 0) mbar_arrive(&sh.prm_bar[blk & 1]);
+      if (lane == 0) mbar_arrive(&sh.prm_bar[filled & 1]);
+      ++filled;
       return rows;
     };
     uint32_t next_rows = fill(0);
     if (p.early) asm volatile("griddepcontrol.wait;" ::: "memory");
-    int it = 0, xc = 0;  // rows, and exchanges of weight sums, so far
+    int it = 0, xc = 0, nb = -1;  // rows and exchanges of weight sums so far; the block's number, as above
     for (int blk = 0; blk < nblk; ++blk) {
       uint32_t mask_rows32 = next_rows;
-      next_rows = fill(blk + 1);  // (over the parameters of block blk - 1, which every warp is done with)
+      nb += mask_rows32 != 0 ? 1 : 0;
+      next_rows = fill(blk + 1);  // (over the parameters of an earlier block, which every warp is done with)
       if (rank == 0) {  // the block's inactive rows
         const int r = row_of(blk * 32 + lane);
         if (r < p.rows && !((mask_rows32 >> lane) & 1u)) {
@@ -909,7 +920,7 @@ __global__ void __launch_bounds__(kHeadThreads, 3) sample_head_kernel(const Head
       for (; mask_rows32; mask_rows32 &= mask_rows32 - 1, ++it) {
         const int kk = __ffs(mask_rows32) - 1;
         const int row = row_of(blk * 32 + kk);
-        const RowParams rp = sh.prm[blk & 1][kk];
+        const RowParams rp = sh.prm[nb & 1][kk];
         const int buf = it & 1;
         const bool fine = wwait(&sh.sum_bar[buf], (uint32_t)(it >> 1) & 1u, false);
         const float M = sh.row_max[buf];
