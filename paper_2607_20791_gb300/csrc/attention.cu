@@ -261,7 +261,6 @@ namespace {
 constexpr size_t kStaticScratchBytes = size_t(8) << 20;  // 8 MiB
 __device__ __align__(256) uint8_t g_attn_scratch[kStaticScratchBytes];
 
-constexpr int kMaxDevices = 64;
 std::mutex g_scratch_mu;
 void* g_scratch_ptr[kMaxDevices] = {};
 

@@ -1412,8 +1412,8 @@ __global__ void __launch_bounds__(AttnCfg<D, NS, QS>::kThreads, 1)
 template <int D, int NS, int QS>
 int launch_attn_cfg(const CUtensorMap& tmK, const CUtensorMap& tmV, const AttnParams& p, int smem_bytes,
                     cudaStream_t st) {
-  static bool done = false;
-  if (int rc = ensure_smem(attn_kernel<D, NS, QS>, kSmemLimit, &done)) return rc;
+  static std::atomic<bool> done[kMaxDevices] = {};
+  if (int rc = ensure_smem(attn_kernel<D, NS, QS>, kSmemLimit, done)) return rc;
   // (its blocks are placed, and set up what needs no input, while the previous kernel finishes)
   const cudaError_t e = launch_dependent(attn_kernel<D, NS, QS>, p.C, AttnCfg<D, NS, QS>::kThreads, smem_bytes, st,
                                          tmK, tmV, p);

@@ -3,6 +3,7 @@
 
 #include <cuda_runtime.h>
 
+#include <atomic>
 #include <cstdarg>
 #include <cstdint>
 #include <cstdio>
@@ -40,13 +41,21 @@ cudaError_t launch_dependent(void (*kernel)(P...), int grid, int block, int smem
   return e == cudaSuccess ? cudaGetLastError() : e;
 }
 
-// Opts a kernel into `bytes` of dynamic shared memory once per process.
+constexpr int kMaxDevices = 64;  // devices whose state is kept (others are asked on every call)
+
+// Opts a kernel into `bytes` of dynamic shared memory on the current device (the
+// attribute is a device's own), once for each: `done`, one flag a device, is the
+// kernel's.
 template <typename Kernel>
-int ensure_smem(Kernel k, int bytes, bool* done) {
-  if (*done) return RGD_OK;
-  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+int ensure_smem(Kernel k, int bytes, std::atomic<bool> (&done)[kMaxDevices]) {
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return cuda_error(e, "cudaGetDevice");
+  std::atomic<bool>* d = dev < kMaxDevices ? &done[dev] : nullptr;
+  if (d && d->load(std::memory_order_acquire)) return RGD_OK;
+  e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
   if (e != cudaSuccess) return cuda_error(e, "cudaFuncSetAttribute");
-  *done = true;
+  if (d) d->store(true, std::memory_order_release);
   return RGD_OK;
 }
 

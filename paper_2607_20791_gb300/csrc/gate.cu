@@ -15,7 +15,6 @@
 #include <climits>
 #include <cmath>
 #include <map>
-#include <mutex>
 #include <vector>
 
 #include "common.h"
@@ -892,11 +891,10 @@ extern "C" int rgd_soft_gate(const rgd_trie* trie, int32_t groups, int32_t rows_
   const int es = dtype == RGD_F32 ? 4 : 2;
   const bool vec = aligned16(probe_logits) && (row_stride * es) % 16 == 0;  // 16-byte vector loads
   constexpr int kDyn = kSoftStages * kSoftChunk;  // chunk buffers (dynamic shared memory)
-  static std::once_flag attr_once;
-  std::call_once(attr_once, [] {
-    cudaFuncSetAttribute(soft_gate_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, kDyn);
-    cudaFuncSetAttribute(soft_gate_kernel<uint16_t>, cudaFuncAttributeMaxDynamicSharedMemorySize, kDyn);
-  });
+  static std::atomic<bool> done[2][kMaxDevices] = {};
+  if (int rc = dtype == RGD_F32 ? ensure_smem(soft_gate_kernel<float>, kDyn, done[0])
+                                : ensure_smem(soft_gate_kernel<uint16_t>, kDyn, done[1]))
+    return rc;
   cudaLaunchConfig_t cfg = {};
   cfg.blockDim = dim3(kSoftThreads);
   cfg.dynamicSmemBytes = kDyn;
