@@ -747,8 +747,9 @@ __global__ void __launch_bounds__(AttnCfg<D, NS, QS>::kThreads, 1)
     // [floor(c T / Ceff), floor((c + 1) T / Ceff)) of T.  With up to 32 groups (more
     // give every block about as many job ends) and more pages than blocks, every job
     // counts p.end_pages more than it has, for the time of its end, so that a block
-    // with more ends gets fewer pages; positions past a job's pages map to its end.  Every position is some block's, so a job's pieces are exactly the blocks
-    // from that of its first page to that of its last.
+    // with more ends gets fewer pages; positions past a job's pages map to its end.
+    // Every position is some block's, so a job's pieces are exactly the blocks from
+    // that of its first page to that of its last.
     const int pages = p.Hkv * __shfl_sync(0xffffffffu, incl, 31);
     const int extra = few && pages > p.C ? p.end_pages : 0;
     const uint32_t some = __ballot_sync(0xffffffffu, few && sum > 0);
@@ -1033,9 +1034,8 @@ __global__ void __launch_bounds__(AttnCfg<D, NS, QS>::kThreads, 1)
     auto wwait = [&](uint64_t* bar, uint32_t parity) {
       return __all_sync(0xffffffffu, wait_or_abort(bar, parity, abort_flag, p.wait_ns));
     };
-    // the set's queries of the job, and of row sel (a suffix page is visible to one row)
-    // a suffix page is visible to the queries of one row, sel; a prompt page to all
-    // (also to the columns past the job's nq: their Q is 0 and nothing reads them)
+    // the set's queries of row sel: a suffix page is visible to them only, a prompt page
+    // to all (also to the columns past the job's nq: their Q is 0 and nothing reads them)
     auto row_mask = [&](int sel) {  // queries sel * gq .. + gq - 1
       const int lo = max(0, sel * p.gq - q0), hi = min(QS, (sel + 1) * p.gq - q0);
       if (hi <= lo) return 0u;

@@ -155,9 +155,9 @@ __global__ void __launch_bounds__(kGateThreads)
 //
 // One thread-block cluster of K CTAs per group (K by the number of groups, see
 // rgd_soft_gate), each CTA taking an equal contiguous share of the probe's logits,
-// copied into shared memory in chunks by bulk copies issued before anything else.  While they are in
-// flight, the children of the probe's trie node (token, node, confirm flag)
-// are read into shared memory -- every trie lookup of the step is then a
+// copied into shared memory in chunks by bulk copies issued before anything else.
+// While they are in flight, the children of the probe's trie node (token, node,
+// confirm flag) are read into shared memory -- every trie lookup of the step is then a
 // shared-memory scan -- and, when the soft branch can be taken at this step,
 // the candidates' keys (logit, token) and the kProbe best of them.  A
 // candidate's rank -- the number of logits above it -- grows along the

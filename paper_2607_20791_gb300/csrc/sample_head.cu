@@ -4,22 +4,26 @@
 //
 // One thread-block cluster of K CTAs (K chosen per call) handles one row at a
 // time and walks the rows cluster by cluster.  A row is read from HBM once: its
-// 16-byte vectors are cut into equal contiguous ranges, one per stream warp of
-// the cluster, and every stream warp streams its range through a ring of
-// shared-memory slots of its own with bulk copies, holding it there until the
-// row's second pass is over.  Pass 1 finds the row's max and lowest-index argmax
-// (each warp sends its own to every CTA of the cluster); probe rows need no
-// more.  Sample rows form the min-p cutoff from the max and, in pass 2, sum the
-// kept weights of every stripe (32 vectors) from shared memory; every slot that
+// 16-byte vectors are cut into K equal contiguous shares, and each CTA's copy warp
+// brings its share into a ring of shared-memory slots of 1024 vectors, one bulk copy
+// each.  A slot is eight stream warps' work, four stripes (32 vectors, one a lane)
+// each, and holds the row until its second pass is over.  Pass 1 finds the row's max
+// and lowest-index argmax (each warp sends its own to every CTA of the cluster);
+// probe rows need no more.  Sample rows form the min-p cutoff from the max and, in
+// pass 2, sum the kept weights of every stripe from shared memory; every slot that
 // pass 2 has finished takes a slot of the cluster's next row at once, so the
 // copies of the next row run behind this row's exchange and second pass.  The
 // draw belongs to a ninth warp per CTA, which works on row i while the stream
-// warps go on with row i + 1: the Philox target u * Z picks CTA, warp and stripe
-// by prefix sums in index order, and that one stripe is read again to find the
-// lane and the element.  Sums are fp32 with compensation (a few ulp, well inside
-// the 1e-6 of Z within which a draw counts as a boundary case); FP64 is slow on
-// this part, so the only fp64 steps are the cutoff's logarithm and the draw's
-// few prefix sums, both off the stream warps' path.
+// warps go on with row i + 1: the Philox target u * Z picks CTA, lane segment and
+// stripe by prefix sums in index order, and that one stripe is read again to find
+// the lane and the element.
+//
+// A stripe's weights (128 or 256) are summed in fp32 by a tree: 7 or 9 roundings one
+// above the other, 8 or 12 in a slot that is not all the row's.  So a stripe's sum is
+// at most 12 x 2^-24 = 7e-7 of itself off, and the cumulative sums no more of Z:
+// inside the 1e-6 of Z within which a draw counts as a boundary case.  From there on
+// sums are 64-bit fixed point, exact in any order; FP64 is slow on this part, and the
+// only fp64 step is the cutoff's logarithm, off the stream warps' path.
 //
 // What bounds it: see launch_head (the split per size) for the measured figures.
 #include <algorithm>
