@@ -210,9 +210,9 @@ int rgd_prefix_decode_attn_noalloc(const rgd_attn_shape* shape, const rgd_bf16* 
  *     step high, 0, 0): u = (word0 >> 8) * 2^-24; token = the smallest i in K
  *     with sum_{j in K, j <= i} w_j > u * sum_K w.
  *   token_out int32 [rows] (-1 for inactive rows and rejected parameters);
- *   kept_count int32 [rows] or NULL: |K| (0 for inactive rows);
+ *   kept_count int32 [rows] or NULL: |K| (0 for inactive and rejected rows);
  *   kept_mask uint8 [rows, vocab] or NULL: 1 where i in K (sample rows only;
- *     rows that are greedy or inactive are not written).
+ *     rows that are greedy, inactive or rejected are not written).
  * is_probe may be NULL (no probe rows); row_active may be NULL (all active).
  * vocab must satisfy vocab * element size <= 2 MiB.  A wait that gives up sets
  * RGD_DEV_WAIT_TIMEOUT in dev_status; outputs of rows then are missing. */

@@ -794,7 +794,9 @@ __global__ void __launch_bounds__(kHeadThreads, 3) sample_head_kernel(const Head
           // ---- pass 2: kept weights; the sum of every stripe and of the warp ----
           const float cut = __fadd_rn(M, rp.theta);  // the min-p cutoff fl32(M + fl32(T ln p_min))
           const float kexp = rp.kexp;
-          uint8_t* mask = p.kept_mask ? p.kept_mask + (int64_t)row * p.vocab : nullptr;
+          // (a rejected row has no kept set: its mask is not written)
+          uint8_t* mask =
+              p.kept_mask && rp.valid && isfinite(M) ? p.kept_mask + (int64_t)row * p.vocab : nullptr;
           const uint32_t hits = mask ? ~0u : __ballot_sync(0xffffffffu, slot_max >= cut);
           const typename V::Cut vc(cut, M, kexp);
           int32_t cnt = 0;

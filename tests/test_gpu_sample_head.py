@@ -139,3 +139,29 @@ def test_steps_change_the_draw(gpu_lib):
         assert dev.token_out.item() == ref.token or ref.boundary
         toks.append(dev.token_out.item())
     assert len(set(toks)) > 4
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("vocab", [40, 4099, 33000])
+def test_rejected_rows_leave_their_mask(gpu_lib, dtype, vocab):
+    # rows with a bad temperature or min-p, or no finite maximum: token -1, nothing
+    # kept, their kept mask untouched; the sampled rows between them as ever
+    import torch
+    inf, nan = float("inf"), float("nan")
+    temps = np.array([1.5, -1.0, nan, inf, 1.5, 1.5, 1.5, 1.5, 1.5], np.float32)
+    minp = np.array([0.1, 0.1, 0.1, 0.1, nan, 1.5, 0.0, 0.1, 0.1], np.float32)
+    logits = np.random.default_rng(vocab).standard_normal((9, vocab)).astype(np.float32)
+    logits[6], logits[7, vocab // 2] = -inf, inf
+    case = workloads.make_head_case("rejected", logits, dtype, np.zeros(9, np.uint8), temps, minp, 3, step=1)
+    dev = device.head_to_device(case, with_mask=True)
+    dev.kept_mask.fill_(9)
+    dev.run()
+    torch.cuda.synchronize()
+    mask, rejected = dev.kept_mask.cpu().numpy(), list(range(1, 8))
+    assert np.all(mask[rejected] == 9)
+    assert np.all(dev.token_out.cpu().numpy()[rejected] == -1) and np.all(dev.kept_count.cpu().numpy()[rejected] == 0)
+    ref = osamp.sample_head(case.logits, dtype, case.is_probe, case.temperature, case.min_p, case.seed, case.step,
+                            case.row_active, rows=[0, 8])
+    for r in (0, 8):
+        assert np.array_equal(mask[r], ref.kept[r].astype(np.uint8))
+        assert dev.token_out[r] == ref.tokens[r] or ref.boundary[r]
