@@ -120,11 +120,15 @@ size_t rgd_prefix_decode_attn_workspace_size(const rgd_attn_shape* shape);
  * Every prompt KV page of a group is read once and attended by all
  * rows_per_group * Hq/Hkv queries of that group and kv head; a row's suffix
  * pages are attended by that row's queries.  The pages of all (group, kv head)
- * jobs are divided evenly over num_ctas persistent blocks; a job split across
- * blocks is merged from its partial results by log-sum-exp.
+ * jobs are divided over num_ctas persistent blocks (evenly, a job's end counting
+ * as some pages where groups are few); a job split across blocks is merged from
+ * its partial results by log-sum-exp.
  *
  *   q                  bf16 [R, Hq, D]
- *   k_pages, v_pages   bf16 [num_pages, Hkv, page_size, D]
+ *   k_pages, v_pages   bf16 [num_pages, Hkv, page_size, D].  Slots past a length in
+ *                      a listed page have no weight, but their V must be finite: a
+ *                      NaN or infinity there (or in another row's suffix) makes
+ *                      outputs of the group and kv head NaN (0 x NaN in the MMA)
  *   prompt_block_table int32 [G, max_prompt_pages]: page ids of prompt tokens
  *                      (token t in page table[t / page_size], slot t % page_size)
  *   prompt_len         int32 [G], 0 <= prompt_len <= max_prompt_pages*page_size
